@@ -332,9 +332,12 @@ typedef struct {
                           /* plane range, secondary and TOF coordinates, sample  */
                           /* length), 1/(P^LM 1)_e and 1/mu_e are stored (40 B   */
                           /* per event); each data update then reads them        */
-                          /* instead of setting the traversals up again.  Same   */
-                          /* per-sample arithmetic as the direct kernel; S_e and */
-                          /* (y+ - y)/mu from the stored reciprocals.  Batches   */
+                          /* instead of setting the traversals up again, walking  */
+                          /* z-pair copies of x (two lanes per voxel plane,       */
+                          /* whatever `group` says).  Same samples and weights as */
+                          /* the direct kernel, summed in another order; S_e and  */
+                          /* (y+ - y)/mu from stored values.  Grids of 2^29       */
+                          /* voxels or more use the direct kernel.  Batches       */
                           /* (lmspdhg_batch_*) run their frames' tables too.     */
                           /* With group = 0 the autotuner also times the direct  */
                           /* event kernel on one subset and keeps the faster     */

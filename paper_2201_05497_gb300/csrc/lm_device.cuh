@@ -49,8 +49,10 @@ __device__ __forceinline__ int sel3i(int k, int a, int b, int c) { return k == 0
 
 // Sets up the traversal; returns false if the LOR has no candidate sample.
 // m: signed TOF bin (ignored unless tofmode == TOF_BIN).
+// stored: the traversal is kept (tables, tiles) rather than used at once; it
+// only chooses which product of the TOF coordinate is rounded first.
 __device__ __forceinline__ bool lor_setup(const Geo& G, int d1, int d2, int m, int tofmode, bool has_yf,
-                                          Lor& L)
+                                          Lor& L, bool stored = false)
 {
     const float* A = G.xtal + 3 * d1;
     const float* B = G.xtal + 3 * d2;
@@ -85,8 +87,11 @@ __device__ __forceinline__ bool lor_setup(const Geo& G, int d1, int d2, int m, i
     L.ub0 = (fmaf(mu0, db, cb) - ob) / hb;
     L.sb = dmu * db / hb;
     L.step = hk * Llen * fabsf(inv);
-    L.tau0 = mu0 * Llen;
-    if (tofmode == TOF_BIN) L.tau0 -= (float)m * G.bin;
+    // spelled out, not left to the compiler's contraction: a sample within an ulp of the 3-sigma cut
+    // must not move in or out of the window when a kernel around this is rearranged
+    L.tau0 = __fmul_rn(mu0, Llen);
+    if (tofmode == TOF_BIN)
+        L.tau0 = stored ? fmaf(mu0, Llen, -__fmul_rn((float)m, G.bin)) : fmaf(-(float)m, G.bin, L.tau0);
     L.dtau = dmu * Llen;
     const int nk = sel3i(k, G.n[0], G.n[1], G.n[2]);
     L.nA = sel3i(ka, G.n[0], G.n[1], G.n[2]);

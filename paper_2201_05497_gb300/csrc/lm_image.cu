@@ -379,7 +379,12 @@ __device__ __forceinline__ void image_tile(const lmh::ImgArgs& A, const PassMode
                     if (have_yf) s += sm.i[tx][ty + q * TR];
                     dz[q] = (float)((double)s * m.fx);
                 } else {
-                    dz[q] = A.acc_pairs ? acc_std[2 * j] + (below ? acc_std[2 * (j - sz) + 1] : 0.0f) : acc_std[j];
+                    if (A.xp != nullptr && !m.init) {
+                        const char* a = (const char*)acc_std + A.lay.at(xx, yy, Tl.z);
+                        dz[q] = *(const float*)a + (below ? *(const float*)(a - A.lay.zs + 4) : 0.0f);
+                    } else {
+                        dz[q] = A.acc_pairs ? acc_std[2 * j] + (below ? acc_std[2 * (j - sz) + 1] : 0.0f) : acc_std[j];
+                    }
                     if (have_yf) dz[q] += sm.f[tx][ty + q * TR];
                 }
             } else {
@@ -396,6 +401,10 @@ __device__ __forceinline__ void image_tile(const lmh::ImgArgs& A, const PassMode
             if (m.data) {
                 if (det) {
                     acci_std[j] = 0ULL;
+                } else if (A.xp != nullptr && !m.init) {
+                    char* a = (char*)acc_std + A.lay.at(xx, yy, Tl.z);
+                    *(float*)a = 0.0f;
+                    if (below) *(float*)(a - A.lay.zs + 4) = 0.0f;
                 } else if (A.acc_pairs) {
                     acc_std[2 * j] = 0.0f;
                     if (below) acc_std[2 * (j - sz) + 1] = 0.0f;
@@ -426,6 +435,12 @@ __device__ __forceinline__ void image_tile(const lmh::ImgArgs& A, const PassMode
             if (kahan) zc[j] = zl;
             x_nxt_std[j] = xn;
             sm.x[r][tx] = xn;
+            if (A.xp != nullptr) {
+                char* p = (char*)A.xp + A.lay.at(xx, yy, Tl.z);
+                *(float*)p = xn;
+                if (below) *(float*)(p - A.lay.zs + 4) = xn;
+                if (Tl.z == A.n[2] - 1) *(float*)(p + 4) = 0.0f;
+            }
         }
     }
     __syncthreads();
@@ -485,8 +500,6 @@ __global__ void __launch_bounds__(256) image_batch_kernel(const lmh::BatchImgArg
 
 constexpr int XHW = 40, XHH = 34;  // x halo box: x0-4 .. x0+35, y0-1 .. y0+32
 constexpr int WBW = 36, WBH = 33;  // w box: x0-4 .. x0+31, y0-1 .. y0+31 (per component)
-constexpr int EW = 33;             // region of w+: x0-1 .. x0+31, y0-1 .. y0+31
-constexpr int EWW = EW * EW;
 constexpr int TP = 33;             // pitch of the transposed tiles
 
 struct TmaLayout {  // byte offsets into dynamic shared memory
@@ -499,15 +512,15 @@ struct TmaLayout {  // byte offsets into dynamic shared memory
     static constexpr int p_wc = 0, p_T = 14336, p_z = p_T + 4096, p_zc = p_z + 4096;
     // data stage: acc_std, acc_yf (u64 when deterministic), x, T, z, zc
     static constexpr int d_as = 0, d_ay = 8192, d_x = 16384, d_T = 20480, d_z = 24576, d_zc = 28672;
-    static constexpr int dbuf = stage + 2 * stage_sz;  // w+ - w (3 x 33 x 33 floats) / transposed acc_yf
-    static constexpr int dbuf_sz = 13184;
+    static constexpr int dbuf = stage + 2 * stage_sz;  // components of w+ - w of neighbours / transposed acc_yf
+    static constexpr int dbuf_sz = 8448;
     static constexpr int xo = dbuf + dbuf_sz;  // transposed x tile
     static constexpr int xo_sz = 4224;
     static constexpr int total = xo + xo_sz;
 };
 static_assert(TmaLayout::p_zc + 4096 <= TmaLayout::stage_sz, "prior stage");
 static_assert(TmaLayout::d_zc + 4096 <= TmaLayout::stage_sz, "data stage");
-static_assert(XHW * XHH * 4 <= TmaLayout::xh_sz && 3 * EWW * 4 <= TmaLayout::dbuf_sz &&
+static_assert(XHW * XHH * 4 <= TmaLayout::xh_sz && (TD + 2) * TD * 4 <= TmaLayout::dbuf_sz &&
                   TD * TP * 8 <= TmaLayout::dbuf_sz && TD * TP * 4 <= TmaLayout::xo_sz,
               "buffers");
 
@@ -703,10 +716,85 @@ __device__ __forceinline__ void store_x_yf(const lmh::ImgArgs& A, const float* X
     }
 }
 
+// Four pairs of voxels x .. x + 3 (x a multiple of 4) at byte address p: two
+// 16-byte halves, of two sectors of a brick or consecutive in a row.
+__device__ __forceinline__ void st_pairs4(char* p, const lmh::PairLay& L, const float* lo, const float* hi)
+{
+    *reinterpret_cast<float4*>(p) = make_float4(lo[0], hi[0], lo[1], hi[1]);
+    *reinterpret_cast<float4*>(p + (L.brick ? 32 : 16)) = make_float4(lo[2], hi[2], lo[3], hi[3]);
+}
+__device__ __forceinline__ void ld_pairs4(const char* p, const lmh::PairLay& L, float* lo, float* hi)
+{
+    const float4 a = *reinterpret_cast<const float4*>(p);
+    const float4 b = *reinterpret_cast<const float4*>(p + (L.brick ? 32 : 16));
+    lo[0] = a.x; hi[0] = a.y; lo[1] = a.z; hi[1] = a.w;
+    lo[2] = b.x; hi[2] = b.y; lo[3] = b.z; hi[3] = b.w;
+}
+// One half (0: first, 4: second) of the four pairs.
+__device__ __forceinline__ void st_halves4(char* p, const lmh::PairLay& L, int half, const float* v)
+{
+    const int o = L.brick ? 32 : 16;
+    *reinterpret_cast<float*>(p + half) = v[0];
+    *reinterpret_cast<float*>(p + 8 + half) = v[1];
+    *reinterpret_cast<float*>(p + o + half) = v[2];
+    *reinterpret_cast<float*>(p + o + 8 + half) = v[3];
+}
+
+// The pair image of a run of slices [zb, ze) at four voxels of slice z (p:
+// their pairs): the pairs of the slice below are complete once this slice's
+// x is known; at the ends of the run the halves that belong to it.
+__device__ __forceinline__ void store_x_pairs(char* p, const lmh::PairLay& L, int z, int zb, int ze, int nz,
+                                              const float* below, const float* xn)
+{
+    const float zero[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (z > zb) st_pairs4(p - L.zs, L, below, xn);
+    else if (z > 0) st_halves4(p - L.zs, L, 4, xn);
+    if (z == nz - 1) st_pairs4(p, L, xn, zero);
+    else if (z == ze - 1) st_halves4(p, L, 0, xn);
+}
+
+__device__ __forceinline__ void ld_quad(const float* p, float* v)
+{
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void st_quad(float* p, const float* v)
+{
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// The prior's dual step at one voxel (same operations as prior_voxel): w+ =
+// v / max(1, |v|/beta), v = w + S K x from the forward differences g (the
+// directional TV takes the part perpendicular to the field f), and K^T's
+// operand w+ - w (directional TV: P (w+ - w)) in d.
+__device__ __forceinline__ void dual_voxel(float sp, float beta, bool dtv, bool hz, const float* f, float gx, float gy,
+                                           float gz, float wx, float wy, float wz, float* o, float* d)
+{
+    if (dtv) dtv_perp(f[0], f[1], f[2], gx, gy, gz);
+    const float vx = fmaf(sp, gx, wx);
+    const float vy = fmaf(sp, gy, wy);
+    const float vz = hz ? fmaf(sp, gz, wz) : 0.0f;
+    const float sc = tv_ball_scale(fmaf(vx, vx, fmaf(vy, vy, vz * vz)), beta);
+    // rounded products (never fused into the differences below), as stored by the plain path
+    o[0] = __fmul_rn(vx, sc);
+    o[1] = __fmul_rn(vy, sc);
+    o[2] = __fmul_rn(vz, sc);
+    d[0] = o[0] - wx;
+    d[1] = o[1] - wy;
+    d[2] = hz ? o[2] - wz : 0.0f;
+    if (dtv) dtv_perp(f[0], f[1], f[2], d[0], d[1], d[2]);
+}
+
 // Fused prior update for slice z of item I (z < I.zb: halo slice, only the
-// z component of w+ - w is kept for the next slice).
+// z component of w+ - w is kept for the next slice).  Each thread owns four
+// voxels of a row (16-byte shared and global accesses: one voxel per access
+// left the pass bound by its instructions); 64 threads also take one point each
+// of the tile's -1 halo (row y0-1: its y component, column x0-1: its x
+// component).  K^T needs the left neighbour's x component (a shuffle) and the
+// y component of the row above (through shared memory).
 __device__ __forceinline__ void prior_slice(const lmh::ImgArgs& A, int wp, uint8_t* sm, int s, int z, int zs,
-                                            const Item& I, float* dprev, float* x_nxt_std, float* x_nxt_yf)
+                                            const Item& I, float* dprev, float* xprev, float* x_nxt_std,
+                                            float* x_nxt_yf)
 {
     const int nx = A.n[0], ny = A.n[1], nz = A.n[2];
     const int64_t V = A.V;
@@ -716,122 +804,117 @@ __device__ __forceinline__ void prior_slice(const lmh::ImgArgs& A, int wp, uint8
     const float* X1 = (const float*)(sm + TmaLayout::xh + ((z + 1 - zs) % 3) * TmaLayout::xh_sz);
     const uint8_t* st = sm + TmaLayout::stage + s * TmaLayout::stage_sz;
     const float* WC = (const float*)(st + TmaLayout::p_wc);
-    float* D = (float*)(sm + TmaLayout::dbuf);
+    float* DY = (float*)(sm + TmaLayout::dbuf);  // y components of rows y0-1 .. y0+31, TD per row
+    float* DX = DY + (TD + 1) * TD;              // x components of column x0-1
     float* XO = (float*)(sm + TmaLayout::xo);
     float* wn = A.w_nxt[wp];
     const float sp = A.s_prior, beta = A.beta;
     const float* xi = A.xi;  // directional TV: the structural field [3][V] (3D grids), else nullptr
-    // w+ = v / max(1, |v|/beta), v = w + S K x, over the tile (4 points per
-    // thread) and its -1 halo (row y0-1 and column x0-1: 65 points), and
-    // D = K^T's operand w+ - w; the directional TV takes the part of the
-    // difference vector perpendicular to the field before v and again of
-    // w+ - w (D = P (w+ - w)), in the order of the event kernel's dual step
-    // the field at the thread's points (4 of the tile, at most one of the
-    // halo), all loads issued before any arithmetic
-    const int lane0 = threadIdx.x & 31, wrow0 = threadIdx.x >> 5, t0 = threadIdx.x;
-    float fxr[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, fyr[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f},
-          fzr[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    if (xi != nullptr) {
+    const bool dtv = xi != nullptr;
+    const int t = threadIdx.x, ty = t >> 3, tx = (t & 7) * 4;
+    const int ix = I.x0 + tx, iy = I.y0 + ty;
+    const bool valid = ix < nx && iy < ny;  // rows are multiples of 4 voxels
+    const int64_t j = ((int64_t)z * ny + iy) * nx + ix;
+    float xc[4], dx[4] = {0.0f, 0.0f, 0.0f, 0.0f}, dy[4] = {0.0f, 0.0f, 0.0f, 0.0f}, dzc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    ld_quad(X0 + (ty + 1) * XHW + tx + 4, xc);
+    if (valid) {
+        const int xb = (ty + 1) * XHW + tx + 4, wb = (ty + 1) * WBW + tx + 4;
+        float f[3][4] = {};
+        if (dtv) {
+            ld_quad(xi + j, f[0]);
+            ld_quad(xi + V + j, f[1]);
+            if (hz) ld_quad(xi + 2 * V + j, f[2]);
+        }
+        float xy[4], xz[4], w[3][4] = {}, o[3][4];
+        const float xr = X0[xb + 4];
+        ld_quad(X0 + xb + XHW, xy);
+        ld_quad(X1 + xb, xz);
+        ld_quad(WC + wb, w[0]);
+        ld_quad(WC + WBW * WBH + wb, w[1]);
+        if (hz) ld_quad(WC + 2 * WBW * WBH + wb, w[2]);
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            int ex, ey;
-            if (k < 4) {
-                ex = lane0 + 1;
-                ey = wrow0 + 8 * k + 1;
-            } else {
-                ex = t0 < EW ? t0 : 0;
-                ey = t0 < EW ? 0 : t0 - EW + 1;
-            }
-            const int ix = I.x0 - 1 + ex, iy = I.y0 - 1 + ey;
-            if ((k < 4 || t0 < 2 * EW - 1) && ix >= 0 && iy >= 0 && ix < nx && iy < ny) {
-                const int64_t j = ((int64_t)z * ny + iy) * nx + ix;
-                fxr[k] = __ldg(xi + j);
-                fyr[k] = __ldg(xi + V + j);
-                if (hz) fzr[k] = __ldg(xi + 2 * V + j);
-            }
+        for (int e = 0; e < 4; ++e) {
+            const float gx = ix + e < nx - 1 ? (e < 3 ? xc[(e + 1) & 3] : xr) - xc[e] : 0.0f;
+            const float gy = iy < ny - 1 ? xy[e] - xc[e] : 0.0f;
+            const float gz = hz ? (z < nz - 1 ? xz[e] - xc[e] : 0.0f) : 0.0f;
+            const float fe[3] = {f[0][e], f[1][e], f[2][e]};
+            float oe[3], de[3];
+            dual_voxel(sp, beta, dtv, hz, fe, gx, gy, gz, w[0][e], w[1][e], w[2][e], oe, de);
+            o[0][e] = oe[0];
+            o[1][e] = oe[1];
+            o[2][e] = oe[2];
+            dx[e] = de[0];
+            dy[e] = de[1];
+            dzc[e] = de[2];
+        }
+        if (own) {
+            st_quad(wn + j, o[0]);
+            st_quad(wn + V + j, o[1]);
+            if (hz) st_quad(wn + 2 * V + j, o[2]);
         }
     }
-    auto wplus = [&](int ex, int ey, bool tile_pt, int k) {
-        const int ix = I.x0 - 1 + ex, iy = I.y0 - 1 + ey;
-        float dx = 0.0f, dy = 0.0f, dzc = 0.0f;
-        if (ix >= 0 && iy >= 0 && ix < nx && iy < ny) {
-            const int xb = ey * XHW + ex + 3;
-            const int wb = ey * WBW + ex + 3;
-            const float xc = X0[xb];
-            const float wx = WC[wb], wy = WC[WBW * WBH + wb];
-            float gx = ix < nx - 1 ? X0[xb + 1] - xc : 0.0f;
-            float gy = iy < ny - 1 ? X0[xb + XHW] - xc : 0.0f;
-            float gz = hz ? (z < nz - 1 ? X1[xb] - xc : 0.0f) : 0.0f;
-            const float fx = fxr[k], fy = fyr[k], fz = fzr[k];
-            if (xi != nullptr) dtv_perp(fx, fy, fz, gx, gy, gz);
-            const float vx = fmaf(sp, gx, wx);
-            const float vy = fmaf(sp, gy, wy);
-            float vz = 0.0f, wz = 0.0f;
-            if (hz) {
-                wz = WC[2 * WBW * WBH + wb];
-                vz = fmaf(sp, gz, wz);
+    st_quad(DY + (ty + 1) * TD + tx, dy);
+    if (t < 2 * TD) {
+        // halo: threads 0-31 the row y0-1, threads 32-63 the column x0-1
+        const bool row = t < TD;
+        const int hx = row ? I.x0 + t : I.x0 - 1, hy = row ? I.y0 - 1 : I.y0 + t - TD;
+        float de[3] = {0.0f, 0.0f, 0.0f};
+        if (hx >= 0 && hy >= 0 && hx < nx && hy < ny) {
+            const int xb = (hy - I.y0 + 1) * XHW + (hx - I.x0 + 4), wb = (hy - I.y0 + 1) * WBW + (hx - I.x0 + 4);
+            const int64_t jh = ((int64_t)z * ny + hy) * nx + hx;
+            float fe[3] = {0.0f, 0.0f, 0.0f}, oe[3];
+            if (dtv) {
+                fe[0] = __ldg(xi + jh);
+                fe[1] = __ldg(xi + V + jh);
+                if (hz) fe[2] = __ldg(xi + 2 * V + jh);
             }
-            const float sc = tv_ball_scale(fmaf(vx, vx, fmaf(vy, vy, vz * vz)), beta);
-            // rounded products (never fused into the differences below), as stored by the plain path
-            const float ox = __fmul_rn(vx, sc), oy = __fmul_rn(vy, sc), oz = __fmul_rn(vz, sc);
-            dx = ox - wx;
-            dy = oy - wy;
-            dzc = hz ? oz - wz : 0.0f;
-            if (xi != nullptr) dtv_perp(fx, fy, fz, dx, dy, dzc);
-            if (own && tile_pt) {
-                const int64_t j = ((int64_t)z * ny + iy) * nx + ix;
-                wn[j] = ox;
-                wn[V + j] = oy;
-                if (hz) wn[2 * V + j] = oz;
-            }
+            const float c = X0[xb];
+            dual_voxel(sp, beta, dtv, hz, fe, hx < nx - 1 ? X0[xb + 1] - c : 0.0f, hy < ny - 1 ? X0[xb + XHW] - c : 0.0f,
+                       hz ? (z < nz - 1 ? X1[xb] - c : 0.0f) : 0.0f, WC[wb], WC[WBW * WBH + wb],
+                       hz ? WC[2 * WBW * WBH + wb] : 0.0f, oe, de);
         }
-        const int p = ey * EW + ex;
-        D[p] = dx;
-        D[EWW + p] = dy;
-        D[2 * EWW + p] = dzc;
-    };
-    {
-        const int lane = threadIdx.x & 31, wrow = threadIdx.x >> 5;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) wplus(lane + 1, wrow + 8 * k + 1, true, k);
-        const int t = threadIdx.x;
-        if (t < EW) wplus(t, 0, false, 4);
-        else if (t < 2 * EW - 1) wplus(0, t - EW + 1, false, 4);
+        if (row) DY[t] = de[1];
+        else DX[t - TD] = de[0];
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31, wrow = threadIdx.x >> 5;
-    const float* Tt = (const float*)(st + TmaLayout::p_T);
-    const float* Zt = (const float*)(st + TmaLayout::p_z);
-    const float* ZCt = (const float*)(st + TmaLayout::p_zc);
+    const float left = __shfl_up_sync(FULL, dx[3], 1);
+    if (own && valid) {
+        float dyb[4], T[4], z0[4], zc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, zh[4], zl[4], xn[4];
+        ld_quad(DY + ty * TD + tx, dyb);
+        const int tq = ty * TD + tx;
+        ld_quad((const float*)(st + TmaLayout::p_T) + tq, T);
+        ld_quad((const float*)(st + TmaLayout::p_z) + tq, z0);
+        if (A.kahan) ld_quad((const float*)(st + TmaLayout::p_zc) + tq, zc);
+        const float d0 = tx == 0 ? DX[ty] : left;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int ty = wrow + 8 * k, tx = lane;
-        const int ix = I.x0 + tx, iy = I.y0 + ty;
-        const int e = (ty + 1) * EW + tx + 1;
-        if (own && ix < nx && iy < ny) {
+        for (int e = 0; e < 4; ++e) {
             // dz = (K^T (w+ - w))_j, component order and signs of prior_dz
             float dz = 0.0f;
-            if (ix < nx - 1) dz -= D[e];
-            if (ix >= 1) dz += D[e - 1];
-            if (iy < ny - 1) dz -= D[EWW + e];
-            if (iy >= 1) dz += D[EWW + e - EW];
+            if (ix + e < nx - 1) dz -= dx[e];
+            if (ix + e >= 1) dz += e > 0 ? dx[(e + 3) & 3] : d0;
+            if (iy < ny - 1) dz -= dy[e];
+            if (iy >= 1) dz += dyb[e];
             if (hz) {
-                if (z < nz - 1) dz -= D[2 * EWW + e];
-                if (z >= 1) dz += dprev[k];
+                if (z < nz - 1) dz -= dzc[e];
+                if (z >= 1) dz += dprev[e];
             }
-            const int t = ty * TD + tx;
-            float zh, zl;
-            const float xn = primal_step(X0[(ty + 1) * XHW + tx + 4], Tt[t], Zt[t], A.kahan ? ZCt[t] : 0.0f, dz,
-                                         A.inv_p_prior, A.kahan != 0, zh, zl);
-            const int64_t j = ((int64_t)z * ny + iy) * nx + ix;
-            A.z[j] = zh;
-            if (A.kahan) A.zc[j] = zl;
-            x_nxt_std[j] = xn;
-            XO[ty * TP + tx] = xn;
+            xn[e] = primal_step(xc[e], T[e], z0[e], zc[e], dz, A.inv_p_prior, A.kahan != 0, zh[e], zl[e]);
         }
-        dprev[k] = hz ? D[2 * EWW + e] : 0.0f;
+        st_quad(A.z + j, zh);
+        if (A.kahan) st_quad(A.zc + j, zl);
+        st_quad(x_nxt_std + j, xn);
+        if (A.xp != nullptr) {
+            store_x_pairs((char*)A.xp + A.lay.at(ix, iy, z), A.lay, z, I.zb, I.ze, nz, xprev, xn);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) xprev[e] = xn[e];
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) XO[ty * TP + tx + e] = xn[e];
+        }
     }
-    if (own) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) dprev[e] = hz ? dzc[e] : 0.0f;
+    if (own && A.xp == nullptr) {
         __syncthreads();
         store_x_yf(A, XO, x_nxt_yf, I, z);
     }
@@ -945,18 +1028,95 @@ __device__ bool tma_item(const lmh::ImgArgs& A, const PassMode& m, int u, int64_
     // a halo slice below the run: the prior needs its w+, paired accumulators their upper halves
     const bool halo = I.zb > 0 && (prior || (A.acc_pairs && !A.det));
     const int zs = halo ? I.zb - 1 : I.zb;
-    float dprev[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    float dprev[4] = {0.0f, 0.0f, 0.0f, 0.0f}, xprev[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     float prev_y[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if (threadIdx.x == 0) issue_slice(A, prior, xcur, wp, sm, 0, zs, zs, I, true, p.bar);
     for (int z = zs, i = 0; z < I.ze; ++z, ++i) {
         const int s = i & 1;
         if (threadIdx.x == 0 && z + 1 < I.ze) issue_slice(A, prior, xcur, wp, sm, s ^ 1, z + 1, zs, I, false, p.bar);
         if (!stage_wait(p, s, A.err)) return false;
-        if (prior) prior_slice(A, wp, sm, s, z, zs, I, dprev, x_nxt_std, x_nxt_yf);
+        if (prior) prior_slice(A, wp, sm, s, z, zs, I, dprev, xprev, x_nxt_std, x_nxt_yf);
         else data_slice(A, m, sm, s, z, I, x_nxt_std, x_nxt_yf, dprev, prev_y);
         __syncthreads();
     }
     return true;
+}
+
+// Data pass of a frame with the table projector (pair accumulator acc_std,
+// pair image xp; grids of the TMA-staged passes: rows and columns multiples
+// of 4): element by element over a slice, four voxels of a row per thread,
+// marching in z so that a voxel's two accumulator halves (its own pair's first,
+// the second of the pair below) and the two halves of the pair image meet
+// in registers.  Neighbouring lanes take the two rows of a brick's sectors.
+// Part `part` of `nparts` blocks; the threads of all parts split the slices
+// into runs so that each has one column to walk.  HBM-bound: 52 bytes per
+// voxel (pair accumulator read and cleared, x, T, z and its compensation
+// read, z, compensation, x and the pair image written).
+struct SliceIn {  // one slice's inputs of a thread
+    float lo[4], hi[4], x[4], T[4], z[4], zc[4];
+};
+
+__device__ __forceinline__ void load_slice(const lmh::ImgArgs& A, const float* xcur, int64_t j, const char* p, SliceIn& s)
+{
+    ld_pairs4(p, A.lay, s.lo, s.hi);
+    ld_quad(xcur + j, s.x);
+    ld_quad(A.T + j, s.T);
+    ld_quad(A.z + j, s.z);
+    if (A.kahan) ld_quad(A.zc + j, s.zc);
+}
+
+__device__ __forceinline__ void data_stream(const lmh::ImgArgs& A, float inv_p, const float* xcur, float* x_nxt,
+                                            int64_t part, int64_t nparts)
+{
+    const int nx = A.n[0], nz = A.n[2], hq = nx / 4;
+    const int64_t sz = (int64_t)nx * A.n[1];
+    const int Q = (int)(sz / 4);
+    const int64_t threads = nparts * blockDim.x;
+    const int64_t runs0 = threads / Q;
+    const int len = runs0 <= 1 ? nz : (runs0 >= nz ? 1 : (int)((nz + runs0 - 1) / runs0));
+    const int64_t items = (int64_t)Q * ((nz + len - 1) / len);
+    const bool kahan = A.kahan != 0;
+    const unsigned zs = A.lay.zs;
+    const float zero[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int64_t it = part * blockDim.x + threadIdx.x; it < items; it += threads) {
+        const int run = (int)(it / Q), c = (int)(it - (int64_t)run * Q);
+        const int zb = run * len, ze = min(nz, zb + len);
+        const int rp = c / (2 * hq), r = c - rp * 2 * hq;
+        const int y = 2 * rp + (r & 1), x = 4 * (r >> 1);
+        int64_t j = zb * sz + (int64_t)y * nx + x;
+        unsigned o = A.lay.at(x, y, zb);
+        char* acc = (char*)A.acc_std;
+        char* xp = (char*)A.xp;
+        SliceIn in, nxt;
+        float prev[4] = {0.0f, 0.0f, 0.0f, 0.0f}, xprev[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (zb > 0) {
+            float lo[4];
+            ld_pairs4(acc + (o - zs), A.lay, lo, prev);  // the second halves of the pairs below
+        }
+        load_slice(A, xcur, j, acc + o, in);
+        for (int z = zb; z < ze; ++z, j += sz, o += zs) {
+            if (z + 1 < ze) load_slice(A, xcur, j + sz, acc + (o + zs), nxt);
+            float zh[4], zl[4], xn[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const float dz = in.lo[v] + prev[v];
+                prev[v] = in.hi[v];
+                xn[v] = primal_step(in.x[v], in.T[v], in.z[v], kahan ? in.zc[v] : 0.0f, dz, inv_p, kahan, zh[v], zl[v]);
+            }
+            st_quad(A.z + j, zh);
+            if (kahan) st_quad(A.zc + j, zl);
+            st_quad(x_nxt + j, xn);
+            // clear: whole pairs inside the run, the halves this run reads at its ends
+            if (z > zb) st_pairs4(acc + (o - zs), A.lay, zero, zero);
+            else if (z > 0) st_halves4(acc + (o - zs), A.lay, 4, zero);
+            if (z == nz - 1) st_pairs4(acc + o, A.lay, zero, zero);
+            else if (z == ze - 1) st_halves4(acc + o, A.lay, 0, zero);
+            store_x_pairs(xp + o, A.lay, z, zb, ze, nz, xprev, xn);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) xprev[v] = xn[v];
+            in = nxt;
+        }
+    }
 }
 
 __device__ __forceinline__ void tma_block_init(uint8_t* sm, int* abort_flag)
@@ -981,6 +1141,10 @@ __global__ void __launch_bounds__(256, 2) image_tma_kernel(const lmh::ImgArgs A)
     const PassMode m = pass_mode(A, u);
     if ((m.prior && A.skip_prior) || (m.data && !m.init && A.skip_data)) return;  // the other pass serves it
     if (blockIdx.x == 0 && threadIdx.x == 0) reset_next_slot(A, u);
+    if (m.data && A.xp != nullptr) {
+        data_stream(A, m.inv_p, A.x_cur, A.x_nxt_std, blockIdx.x, gridDim.x);
+        return;
+    }
     const int64_t n = tma_items(A);
     for (int64_t it = blockIdx.x; it < n; it += gridDim.x)
         if (!tma_item(A, m, u, it, A.xcur, A.x_nxt_std, A.x_nxt_yf, sm, p)) break;
@@ -1010,6 +1174,10 @@ __global__ void __launch_bounds__(256, 2) image_tma_batch_kernel(const lmh::Batc
         const int64_t lt = t - (int64_t)s * B.tiles_per_slot;
         const PassMode m = pass_mode(A, B.u);
         if (lt == 0 && threadIdx.x == 0) reset_next_slot(A, B.u);
+        if (m.data && A.xp != nullptr) {
+            data_stream(A, m.inv_p, A.xbuf[par], A.xbuf[par ^ 1], lt, B.tiles_per_slot);
+            continue;
+        }
         if (!tma_item(A, m, B.u, lt, par, A.xbuf[par ^ 1], A.xbuf_yf[par ^ 1], sm, p)) break;
     }
 }
@@ -1583,7 +1751,9 @@ void launch_image_tma(const ImgArgs& a, cudaStream_t st)
     std::memset(&g, 0, sizeof(g));
     for (int d = 0; d < 3; ++d) g.n[d] = a.n[d];
     const int64_t items = tma_items_host(&g, a.zlen);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(items, 2 * (int64_t)num_sms()));
+    // (the data pass of a table frame splits the slices over whatever blocks there are)
+    const int grid =
+        a.xp ? 2 * num_sms() : (int)std::max<int64_t>(1, std::min<int64_t>(items, 2 * (int64_t)num_sms()));
     image_tma_kernel<<<grid, 256, TmaLayout::total, st>>>(a);
     count_launch();
 }

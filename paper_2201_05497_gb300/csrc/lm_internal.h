@@ -183,7 +183,7 @@ struct EvArgs {
     const float* xbyf[2];
     unsigned* maxbits_base;
     int prior_fused;            // 1: the prior's dual step runs inside the TMA image pass instead
-    int prior_only;             // 1: data selections are left to the tile-binned projector
+    int prior_only;             // 1: data selections are left to the tile-binned or the table projector
     int acc_pairs;              // 1: acc_std / acc_yf hold (voxel j, voxel j + nx*ny) float pairs
     const float* xi;            // directional TV field [ndim][V], or nullptr (TV)
     float* dtv_d;               // directional TV: P (w+ - w) of the prior's dual step [ndim][V], or nullptr
@@ -306,6 +306,20 @@ void tile_attributes();
 int launch_tile_update(const TileArgs& A, bool two_d, cudaStream_t st);
 
 // ---- traversal-table data update (lm_table.cu) ----
+// Where the pair of voxel (x, y, z) lies in the table projector's pair images
+// (byte offsets, modulo 2^32): X(x) + Y(y) + z zs with X(i) = i x1 + (i & 2) x2 +
+// (i & 1) x3.  Rows: x2 = x3 = y2 = y3 = 0.  Bricks: 4 x 4 pairs (one 128-byte
+// line) of 2 x 2 sectors.  Shared by the event kernels and the image passes.
+struct PairLay {
+    unsigned x1, x2, x3, y1, y2, y3, zs;
+    int brick;
+    __host__ __device__ unsigned at(unsigned x, unsigned y, unsigned z) const
+    {
+        return x * x1 + (x & 2u) * x2 + (x & 1u) * x3 + y * y1 + (y & 2u) * y2 + (y & 1u) * y3 + z * zs;
+    }
+};
+PairLay pair_layout(const lm_grid* g, bool rows);  // rows: no bricks even where the grid allows them
+
 // Per event (subset-contiguous order): the traversal of reading 1,
 // 1/(P^LM 1)_e and 1/mu_e, computed once per state.
 struct TravLayout {
@@ -318,18 +332,17 @@ struct TabArgs {
     lmk::Geo G;
     // table
     const float4* r0;      // (ua0, sa, ub0, sb)
-    const float4* r1;      // (tau0, dtau, step, 1/(P^LM 1)_e)
-    const int2* meta;      // (i0 | cnt << 15 | k << 30, bits of 1/mu_e); cnt = 0: inert event
+    const float4* r1;      // (tau0, dtau, step, 1/(P^LM 1)_e); step < 0: every sample's neighbours are in the grid
+    const int2* meta;      // (i0 | cnt << 15 | k << 30, bits of (float) mu_e); cnt = 0: inert event
     // events
     const float* corr;
     const float* contam;
     const uint16_t* mu;
     float* y;
-    // images: the x the update gathers from, both layouts; z-paired accumulators (see EvArgs)
-    const float* x_std;
-    const float* x_yf;
-    float* acc_std;
-    float* acc_yf;
+    // images as z pairs (voxel j, voxel j + nx*ny): the x the events read, the accumulator
+    const float* xp;
+    float* acc;
+    PairLay lay;
     const float* tof_tab;  // TOF_TAB_N + 1 floats
     // selection
     const uint16_t* seq;
@@ -338,12 +351,7 @@ struct TabArgs {
     int n_subsets;
     int64_t e_begin, e_end;  // used when seq == nullptr
     float gamma_rho;
-    unsigned long long* queue;
-    unsigned* done;
-    int phase;             // 0: x-principal events only, 1: the others, -1: all
-    // batched epochs: the image of update u is in buffer u & 1
-    const float* xs[2];
-    const float* xyfs[2];
+    float* out;            // EV_FWD: the projections
 };
 
 // The data updates of every active frame of a batch (frames with tables).
@@ -354,18 +362,16 @@ struct BatchTabArgs {
     int seq_stride;
     int cap;
     int u;
-    unsigned long long* queue;  // self-resetting work counter
-    unsigned* done;
     const float* tof_tab;       // the batch's TOF table
     float tof_W;
 };
-int launch_table_batch(const BatchTabArgs& b, int variant, int grid, cudaStream_t st);
+int launch_table_batch(const BatchTabArgs& b, cudaStream_t st);
 int trav_build(const lmk::Geo& G, const lm_events& ev, const uint16_t* mu, const float* tof_tab,
                const TravLayout& L, char* base, cudaStream_t st);
-// variant: the lane-group width 8, 16 or 32 (32 compiled for 3 resident
-// blocks per SM), or 33 (width 32 compiled for 4 blocks per SM)
-int launch_table_update(const TabArgs& a, int variant, int grid, cudaStream_t st);
-int table_grid(int variant);
+// xp = x as z pairs (voxel j, voxel j + nx*ny)
+void launch_pair_image(const lm_grid* g, const PairLay& P, const float* x, float* xp, cudaStream_t st);
+// mode: EV_DATA or EV_FWD (out[e] = c_e J_e x)
+int launch_table(int mode, const TabArgs& a, cudaStream_t st);
 
 // ---- image kernels (lm_image.cu) ----
 void launch_transpose_to_yf(const lm_grid* g, const float* src, float* dst, cudaStream_t st);
@@ -441,6 +447,9 @@ struct ImgArgs {
     const float* dtv_d;    // directional TV: P (w+ - w) from the dual step, or nullptr (formed here)
     int skip_prior;        // 1: return at once when the update is a prior update
     int skip_data;         // 1: return at once when the update is a data update
+    float* xp;             // z pairs of x for the table projector (written instead of the y-fastest copy; the data
+                           // updates' accumulator is then acc_std alone), or nullptr
+    PairLay lay;           // where xp and that accumulator hold a voxel's pair
 };
 
 struct BatchImgArgs {

@@ -666,7 +666,7 @@ __global__ void __launch_bounds__(256, G == 8 ? 2 : 3) ev_batch_kernel(const lmh
                 kind = 1;
                 eb = A.sub_off[sel];
                 ee = A.sub_off[sel + 1];
-                items = (ee - eb + A.chunk - 1) / A.chunk;
+                items = A.prior_only ? 0 : (ee - eb + A.chunk - 1) / A.chunk;
                 if (T::back_fx) {
                     const float vmax = __uint_as_float(A.maxbits_base[sidx]);
                     fxs = ldexpf(1.0f, fx_exponent(vmax, ee - eb, A.stepmax));

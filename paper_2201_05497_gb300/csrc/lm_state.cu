@@ -63,6 +63,7 @@ struct lm_state_s {
     int zlen;         // z slices per TMA work item
     bool table;       // data updates from the traversal table (lm_table.cu)
     TravLayout tv;    // its layout in the caller's buffer
+    PairLay lay;      // layout of its pair images
     char* tv_base;
     bool tiled;       // data updates by the tile-binned projector
     TileArgs ta;      // its per-frame tables (pointers into the caller's tile buffer)
@@ -71,12 +72,9 @@ struct lm_state_s {
     int64_t n_segments;
     size_t scr_bytes;
     int grid_ev, grid_fx, chunk;
-    int grid_tab;       // blocks of the traversal-table kernel
-    int tab_variant;    // its compiled variant (launch_table_update)
-    bool tab_split;     // one launch per principal-axis family (else one for all)
     int group;          // lanes per event of the event kernels
-    double tune_ms[3];  // autotuner: forward projection of subset 0 with 8, 16, 32 lanes
-    double tune_table_ms, tune_direct_ms;  // data update of subset 0: best table / direct variant
+    double tune_ms[3];  // autotuner: subset 0 with 8, 16, 32 lanes (direct kernel)
+    double tune_table_ms, tune_direct_ms;  // data update of subset 0: table kernel / best direct width
     cudaStream_t cap_stream;
     cudaGraphExec_t exec;
     bool have_graph;
@@ -254,11 +252,21 @@ ImgArgs base_img_args(const lm_state* st)
     a.zlen = st->zlen;
     a.xi = st->P.xi;
     a.dtv_d = st->dtvd;
+    if (st->table) {
+        a.acc_yf = nullptr;
+        a.xp = st->xyf[0];
+        a.lay = st->lay;
+    }
     return a;
 }
 
-// Arguments of the traversal-table data update of update u (x in buffer cur).
-TabArgs base_tab_args(const lm_state* st, int cur)
+// The pair image of x that the table projector reads (voxel j, voxel
+// j + nx*ny): it takes the place of the two y-fastest copies of the direct
+// kernel (adjacent in the state buffer); its accumulator is acc_std alone.
+float* pair_image(const lm_state* st) { return st->xyf[0]; }
+
+// Arguments of the traversal-table kernels.
+TabArgs base_tab_args(const lm_state* st)
 {
     TabArgs t;
     std::memset(&t, 0, sizeof(t));
@@ -270,17 +278,13 @@ TabArgs base_tab_args(const lm_state* st, int cur)
     t.contam = st->contam;
     t.mu = st->mu;
     t.y = st->y;
-    t.x_std = st->x[cur];
-    t.x_yf = st->xyf[cur];
-    t.acc_std = st->acc_std;
-    t.acc_yf = st->acc_yf;
+    t.xp = pair_image(st);
+    t.acc = st->acc_std;
+    t.lay = st->lay;
     t.tof_tab = st->tof_tab;
     t.sub_off = st->sub_off;
     t.n_subsets = st->n;
     t.gamma_rho = (float)(st->gamma * (double)st->P.rho);
-    t.queue = st->queue;
-    t.done = st->done;
-    t.phase = -1;
     return t;
 }
 
@@ -346,17 +350,11 @@ int launch_event_part(lm_state* st, int u, int cur, int slot, cudaStream_t s)
             LM_CHECK(rc == LM_OK, rc, "prior update launch failed");
         }
     } else if (st->table) {
-        // the table kernel, one launch per principal-axis family so that one
-        // image layout and one accumulator layout share L2 (both return at
-        // once on a prior update)
-        TabArgs t = base_tab_args(st, cur);
+        // the table kernel (returns at once on a prior update)
+        TabArgs t = base_tab_args(st);
         t.seq = st->seq;
         t.u = u;
-        int rc = LM_OK;
-        for (int ph = st->tab_split ? 0 : -1; ph < (st->tab_split ? 2 : 0) && rc == LM_OK; ++ph) {
-            t.phase = ph;
-            rc = launch_table_update(t, st->tab_variant, st->grid_tab, s);
-        }
+        int rc = launch_table(EV_DATA, t, s);
         LM_CHECK(rc == LM_OK, rc, "data update launch failed");
         if (!tma_fuses_prior(st)) {
             // the image pass needs w+ (and D) from the event kernel's prior branch
@@ -400,7 +398,7 @@ int launch_image_part(lm_state* st, int u, int cur, int nxt, int slot0, cudaStre
     im.u = u;
     im.x_cur = st->x[cur];
     im.x_nxt_std = st->x[nxt];
-    im.x_nxt_yf = st->xyf[nxt];
+    im.x_nxt_yf = st->table ? nullptr : st->xyf[nxt];
     // scale slots: update u reads slot (slot0 + u) & 1, its pass clears the other one
     im.slot0 = slot0;
     im.xcur = cur;
@@ -456,10 +454,11 @@ int init_image_pass(lm_state* st, const float* x0, cudaStream_t s)
 {
     ImgArgs im = base_img_args(st);
     im.mode = IP_INIT;
+    im.acc_yf = st->acc_yf;  // the initialisation ran the direct kernel: both its accumulators
     im.x_cur = x0;
     im.x_keep = st->x[1];
     im.x_nxt_std = st->x[0];
-    im.x_nxt_yf = st->xyf[0];
+    im.x_nxt_yf = st->table ? nullptr : st->xyf[0];
     launch_image_pass(im, s);
     if (st->has_res) {
         int rc = res_fwd(st, st->x[0], s);
@@ -528,6 +527,8 @@ int init_iteration(lm_state* st, const float* x0, cudaStream_t s)
     a.chunk = chunk_for(st->N, st->grid_ev);  // all N events, not one subset
     if (st->N > 0) {
         if (!st->det) {
+            // (the direct kernel for every projector: it sums all events at once, and its two
+            // accumulators, one per principal-axis family, keep the float sums short)
             a.acc_std = st->acc_std;
             a.acc_yf = st->acc_yf;
             rc = launch_events(EV_YINIT, st->two_d, a, st->grid_ev, s);
@@ -616,137 +617,72 @@ int autotune_group(lm_state* st, cudaStream_t s)
     return LM_OK;
 }
 
-// Autotuner of the traversal-table path: times the data update of subset 0
-// (from the x of the first update) with 8, 16 and 32 lanes per event, three
-// runs each (the first warms the caches), restoring the subset's duals
-// before every run; the accumulators are cleared afterwards, so the state is
-// as it was.
-int autotune_table(lm_state* st, cudaStream_t s)
+// Autotuner of the traversal-table path, before the initialisation: times
+// the data update of subset 0 (from x0, with duals 0) by the direct event
+// kernel with 8, 16 and 32 lanes per event (unless the caller keeps the
+// table) and by the table kernel, three runs each (the first warms the
+// caches).  The projector with the shorter data update stays; the
+// initialisation clears what the runs left in y and the accumulators.
+int autotune_table(lm_state* st, const float* x0, cudaStream_t s)
 {
     st->tune_ms[0] = st->tune_ms[1] = st->tune_ms[2] = 0.0;
     const int64_t b0 = st->sub_off_h[0], n0 = st->sub_off_h[1] - st->sub_off_h[0];
     if (n0 <= 0) return LM_OK;
-    float* ysave = st->scr;  // the per-event scratch holds N floats
-    LM_CUDA(cudaMemcpyAsync(ysave, st->y + b0, (size_t)n0 * 4, cudaMemcpyDeviceToDevice, s));
-    TabArgs t = base_tab_args(st, st->xpar);
-    t.e_begin = b0;
-    t.e_end = b0 + n0;
+    st->gamma = st->P.gamma > 0.0f ? (double)st->P.gamma : 1.0;  // any step does for the timing
+    LM_CUDA(cudaMemsetAsync(st->queue, 0, 16, s));
+    LM_CUDA(cudaMemsetAsync(st->done, 0, 16, s));
     cudaEvent_t e0, e1;
     LM_CUDA(cudaEventCreate(&e0));
     LM_CUDA(cudaEventCreate(&e1));
-    // variants: widths 8, 16, 32 (3 blocks per SM) and 32 (4 blocks per SM)
-    const int variants[4] = {8, 16, 32, 33};
-    double ms[4] = {0.0, 0.0, 0.0, 0.0};
-    double best = 1e30;
-    int best_v = 32, rc = LM_OK;
-    for (int w = 0; w < 4 && rc == LM_OK; ++w) {
-        float tot = 0.0f;
+    int rc = LM_OK;
+    // mean of the second and third of three runs (ms)
+    auto time3 = [&](auto&& launch) {
+        double tot = 0.0;
         for (int rep = 0; rep < 3 && rc == LM_OK; ++rep) {
-            cudaMemcpyAsync(st->y + b0, ysave, (size_t)n0 * 4, cudaMemcpyDeviceToDevice, s);
+            cudaMemsetAsync(st->y + b0, 0, (size_t)n0 * 4, s);
             cudaEventRecord(e0, s);
-            rc = launch_table_update(t, variants[w], table_grid(variants[w]), s);
+            rc = launch();
             cudaEventRecord(e1, s);
             cudaEventSynchronize(e1);
             float m = 0.0f;
             cudaEventElapsedTime(&m, e0, e1);
-            if (rep > 0) tot += m;
+            if (rep > 0) tot += m / 2.0;
         }
-        ms[w] = tot / 2.0;
-        if (ms[w] < best) {
-            best = ms[w];
-            best_v = variants[w];
+        return tot;
+    };
+    double direct_ms = 1e30;
+    const int widths[3] = {8, 16, 32};
+    st->group = 32;
+    launch_transpose_to_yf(&st->g, x0, st->xyf[1], s);
+    for (int w = 0; w < 3 && !st->P.trav_keep && rc == LM_OK; ++w) {
+        EvArgs a = base_ev_args(st);
+        a.group = widths[w];
+        a.x_std = x0;
+        a.x_yf = st->xyf[1];
+        a.acc_std = st->acc_std;
+        a.acc_yf = st->acc_yf;
+        a.e_begin = b0;
+        a.e_end = b0 + n0;
+        const int grid = ev_grid_g(EV_DATA, st->two_d, widths[w]);
+        a.chunk = chunk_for(n0, grid);
+        st->tune_ms[w] = time3([&] { return launch_events(EV_DATA, st->two_d, a, grid, s); });
+        if (st->tune_ms[w] < direct_ms) {
+            direct_ms = st->tune_ms[w];
+            st->group = widths[w];  // the direct kernel's width, should it be used
         }
     }
-    // the chosen variant with the principal-axis families in one launch
-    // instead of two
-    double one = 0.0;
-    t.phase = -1;
-    for (int rep = 0; rep < 3 && rc == LM_OK; ++rep) {
-        cudaMemcpyAsync(st->y + b0, ysave, (size_t)n0 * 4, cudaMemcpyDeviceToDevice, s);
-        cudaEventRecord(e0, s);
-        rc = launch_table_update(t, best_v, table_grid(best_v), s);
-        cudaEventRecord(e1, s);
-        cudaEventSynchronize(e1);
-        float m = 0.0f;
-        cudaEventElapsedTime(&m, e0, e1);
-        if (rep > 0) one += m / 2.0;
-    }
-    double two = 0.0;
-    for (int rep = 0; rep < 3 && rc == LM_OK; ++rep) {
-        cudaMemcpyAsync(st->y + b0, ysave, (size_t)n0 * 4, cudaMemcpyDeviceToDevice, s);
-        cudaEventRecord(e0, s);
-        for (int ph = 0; ph < 2 && rc == LM_OK; ++ph) {
-            t.phase = ph;
-            rc = launch_table_update(t, best_v, table_grid(best_v), s);
-        }
-        cudaEventRecord(e1, s);
-        cudaEventSynchronize(e1);
-        float m = 0.0f;
-        cudaEventElapsedTime(&m, e0, e1);
-        if (rep > 0) two += m / 2.0;
-    }
-    st->tab_split = two <= one;
+    launch_pair_image(&st->g, st->lay, x0, pair_image(st), s);
+    TabArgs t = base_tab_args(st);
+    t.e_begin = b0;
+    t.e_end = b0 + n0;
+    const double table_ms = time3([&] { return launch_table(EV_DATA, t, s); });
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) return rc;
-    st->tune_ms[0] = ms[0];
-    st->tune_ms[1] = ms[1];
-    st->tune_ms[2] = std::min(ms[2], ms[3]);
-    LM_CUDA(cudaMemcpyAsync(st->y + b0, ysave, (size_t)n0 * 4, cudaMemcpyDeviceToDevice, s));
-    LM_CUDA(cudaMemsetAsync(st->acc_std, 0, 2 * (size_t)st->V * 4, s));
-    LM_CUDA(cudaMemsetAsync(st->acc_yf, 0, 2 * (size_t)st->V * 4, s));
-    st->tab_variant = best_v;
-    const int best_g = best_v == 33 ? 32 : best_v;
-    st->group = best_g;
-    // the direct event kernel on the same subset: the projector with the shorter data update stays
-    // (unless the caller keeps the table)
-    const double table_ms = std::min(one, two);
-    double direct_ms = 1e30;
-    int direct_g = 32;
-    if (!st->P.trav_keep) {
-        cudaEvent_t d0, d1;
-        LM_CUDA(cudaEventCreate(&d0));
-        LM_CUDA(cudaEventCreate(&d1));
-        const int widths[3] = {8, 16, 32};
-        for (int w = 0; w < 3 && rc == LM_OK; ++w) {
-            EvArgs a = base_ev_args(st);
-            a.group = widths[w];
-            a.x_std = st->x[st->xpar];
-            a.x_yf = st->xyf[st->xpar];
-            a.acc_std = st->acc_std;
-            a.acc_yf = st->acc_yf;
-            a.e_begin = b0;
-            a.e_end = b0 + n0;
-            a.chunk = chunk_for(n0, ev_grid_g(EV_DATA, st->two_d, widths[w]));
-            double tot = 0.0;
-            for (int rep = 0; rep < 3 && rc == LM_OK; ++rep) {
-                cudaMemcpyAsync(st->y + b0, ysave, (size_t)n0 * 4, cudaMemcpyDeviceToDevice, s);
-                cudaEventRecord(d0, s);
-                rc = launch_events(EV_DATA, st->two_d, a, ev_grid_g(EV_DATA, st->two_d, widths[w]), s);
-                cudaEventRecord(d1, s);
-                cudaEventSynchronize(d1);
-                float m = 0.0f;
-                cudaEventElapsedTime(&m, d0, d1);
-                if (rep > 0) tot += m / 2.0;
-            }
-            if (tot < direct_ms) {
-                direct_ms = tot;
-                direct_g = widths[w];
-            }
-        }
-        cudaEventDestroy(d0);
-        cudaEventDestroy(d1);
-        if (rc) return rc;
-        LM_CUDA(cudaMemcpyAsync(st->y + b0, ysave, (size_t)n0 * 4, cudaMemcpyDeviceToDevice, s));
-        LM_CUDA(cudaMemsetAsync(st->acc_std, 0, 2 * (size_t)st->V * 4, s));
-        LM_CUDA(cudaMemsetAsync(st->acc_yf, 0, 2 * (size_t)st->V * 4, s));
-    }
     st->tune_table_ms = table_ms;
     st->tune_direct_ms = st->P.trav_keep ? 0.0 : direct_ms;
-    if (!st->P.trav_keep && direct_ms < table_ms) {
-        st->table = false;
-        st->group = direct_g;
-    }
+    if (direct_ms < table_ms) st->table = false;
+    else st->group = 32;  // for what the direct kernel still does (the initialisation)
     return LM_OK;
 }
 
@@ -988,6 +924,7 @@ int lmspdhg_create(lm_state** out, const lm_scanner* sc, const lm_grid* grid, co
         rc = build_table(st, s);
         if (rc) return fail(rc);
         st->table = true;
+        st->lay = pair_layout(grid, st->shard);  // (event sharding exchanges the accumulator in rows)
     }
     if (P.knorm > 0.0) {
         st->knorm = P.knorm;
@@ -1003,15 +940,19 @@ int lmspdhg_create(lm_state** out, const lm_scanner* sc, const lm_grid* grid, co
     st->grid_fx = ev_grid(EV_BACK_FX, st->two_d);
     st->chunk = choose_chunk(st);
     st->group = (P.group == 8 || P.group == 16 || P.group == 32) ? P.group : 16;
-    rc = init_iteration(st, x0, s);
-    if (rc) return fail(rc);
-    if (P.group == 0) {
-        rc = st->table ? autotune_table(st, s) : autotune_group(st, s);
+    const bool tune_table = st->table && P.group == 0;
+    if (tune_table) {
+        rc = autotune_table(st, x0, s);
         if (rc) return fail(rc);
     }
-    if (P.group != 0) {
-        st->tab_variant = st->group;
-        st->tab_split = true;
+    const int tuned_group = st->group;
+    if (tune_table) st->group = 16;  // the first initialisation runs the default width
+    rc = init_iteration(st, x0, s);
+    if (rc) return fail(rc);
+    st->group = tuned_group;
+    if (P.group == 0 && !tune_table) {
+        rc = autotune_group(st, s);
+        if (rc) return fail(rc);
     }
     st->gate = nullptr;
     {
@@ -1026,7 +967,6 @@ int lmspdhg_create(lm_state** out, const lm_scanner* sc, const lm_grid* grid, co
         st->persist = fits && P.epoch_kernel == 2;
         st->grid_persist = st->persist ? persist_grid(st->group) : 0;
     }
-    st->grid_tab = st->table ? table_grid(st->tab_variant) : 0;
     // the event kernels run with as many resident blocks as the chosen width allows
     st->grid_ev = ev_grid_g(st->det ? EV_DATA_FX1 : EV_DATA, st->two_d, st->group);
     st->grid_fx = ev_grid_g(EV_BACK_FX, st->two_d, st->group);
@@ -1283,7 +1223,21 @@ int lmspdhg_objective_parts_fp64(lm_state* st, double* out4, void* stream)
         a.queue = nullptr;
         a.done = nullptr;
         a.chunk = 32;
-        int rc = launch_events(EV_FWD, st->two_d, a, ev_grid_g(EV_FWD, st->two_d, st->group), s);
+        int rc;
+        if (st->table) {
+            // the pair image of that x goes to the accumulator the table projector leaves unused
+            launch_pair_image(&st->g, st->lay, st->x[xb], st->acc_yf, s);
+            TabArgs t = base_tab_args(st);
+            t.xp = st->acc_yf;
+            t.e_begin = 0;
+            t.e_end = st->N;
+            t.out = p;
+            rc = launch_table(EV_FWD, t, s);
+            // (event sharding folds both accumulators: the unused one stays zero)
+            if (st->shard) LM_CUDA(cudaMemsetAsync(st->acc_yf, 0, 2 * (size_t)st->V * 4, s));
+        } else {
+            rc = launch_events(EV_FWD, st->two_d, a, ev_grid_g(EV_FWD, st->two_d, st->group), s);
+        }
         LM_CHECK(rc == LM_OK, rc, "objective projection failed");
         if (st->has_res) {
             // the accumulators must be zero at the next update
@@ -1444,7 +1398,6 @@ struct BatchCfg {
     int n, n_det, group, zlen;
     bool two_d, det, kahan, tma;
     bool table;       // frames with traversal tables (the batch's data updates from them)
-    int tab_variant;
 };
 
 struct lm_batch_s {
@@ -1514,7 +1467,6 @@ BatchCfg cfg_of(const lm_state* st)
     c.kahan = st->kahan;
     c.tma = st->tma;
     c.table = st->table;
-    c.tab_variant = st->tab_variant;
     return c;
 }
 
@@ -1525,8 +1477,7 @@ bool same_config(const BatchCfg& a, const lm_state* st)
         if (a.g.n[d] != b.g.n[d]) return false;
     return a.n == b.n && a.two_d == b.two_d && a.det == b.det && a.kahan == b.kahan && a.tof.n_bins == b.tof.n_bins &&
            a.tof.sigma_mm == b.tof.sigma_mm && a.tof.bin_mm == b.tof.bin_mm && a.tof.n_sigma == b.tof.n_sigma &&
-           a.n_det == b.n_det && a.group == b.group && a.tma == b.tma && a.zlen == b.zlen && a.table == b.table &&
-           (!a.table || a.tab_variant == b.tab_variant);
+           a.n_det == b.n_det && a.group == b.group && a.tma == b.tma && a.zlen == b.zlen && a.table == b.table;
 }
 
 void fill_slot(lm_batch* b, int s, lm_state* st)
@@ -1543,6 +1494,7 @@ void fill_slot(lm_batch* b, int s, lm_state* st)
     a.xbyf[0] = st->xyf[0];
     a.xbyf[1] = st->xyf[1];
     a.maxbits_base = st->maxbits;
+    a.prior_only = st->table ? 1 : 0;  // the table kernel runs the data updates
     if (!st->det) {
         a.acc_std = st->acc_std;
         a.acc_yf = st->acc_yf;
@@ -1558,21 +1510,17 @@ void fill_slot(lm_batch* b, int s, lm_state* st)
     im.slot0 = 0;
     im.xbuf[0] = st->x[0];
     im.xbuf[1] = st->x[1];
-    im.xbuf_yf[0] = st->xyf[0];
-    im.xbuf_yf[1] = st->xyf[1];
+    if (!st->table) {
+        im.xbuf_yf[0] = st->xyf[0];
+        im.xbuf_yf[1] = st->xyf[1];
+    }
     im.wpar_w = st->wpar;
     im.wbase = st->wbase;
     b->h_ev[s] = a;
     b->h_im[s] = im;
     if (st->table) {
-        TabArgs t = base_tab_args(st, 0);
+        TabArgs t = base_tab_args(st);
         t.seq = nullptr;  // the batch reads the frames' selections itself
-        t.queue = nullptr;
-        t.done = nullptr;
-        for (int k = 0; k < 2; ++k) {
-            t.xs[k] = st->x[k];
-            t.xyfs[k] = st->xyf[k];
-        }
         b->h_tab[s] = t;
     }
 }
@@ -1608,11 +1556,8 @@ int launch_batch_epoch(lm_batch* b, cudaStream_t s)
     bt.seqs = b->d_seqs;
     bt.seq_stride = count;
     bt.cap = b->cap;
-    bt.queue = b->d_queue;
-    bt.done = (unsigned*)(b->d_queue + 1);
     bt.tof_tab = b->d_tof;
     bt.tof_W = r.W;
-    const int g_tab = r.table ? table_grid(r.tab_variant) : 0;
     const int g_ev = ev_batch_grid(r.det ? EV_DATA_FX1 : EV_DATA, r.two_d, r.group);
     const int g_fx = ev_batch_grid(EV_BACK_FX, r.two_d, r.group);
     const int g_im = r.tma ? image_tma_batch_grid(&r.g, b->cap) : image_batch_grid(&r.g, b->cap);
@@ -1621,9 +1566,11 @@ int launch_batch_epoch(lm_batch* b, cudaStream_t s)
         bi.u = u;
         bt.u = u;
         int rc;
-        if (r.table && r.tma) {
-            // data updates from the frames' traversal tables (the prior's dual step is in the image pass)
-            rc = launch_table_batch(bt, r.tab_variant, g_tab, s);
+        if (r.table) {
+            // data updates from the frames' traversal tables; without TMA-staged passes the prior's
+            // dual step runs in the event kernel (it is in the image pass otherwise)
+            rc = launch_table_batch(bt, s);
+            if (!rc && !r.tma) rc = launch_events_batch(EV_DATA, r.two_d, r.group, be, g_ev, s);
         } else if (!r.det) {
             rc = launch_events_batch(EV_DATA, r.two_d, r.group, be, g_ev, s);
         } else {

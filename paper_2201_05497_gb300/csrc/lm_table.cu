@@ -3,33 +3,29 @@
 // divided by mu) from a stored traversal table.
 //
 // The direct event kernel (lm_project.cu) sets up every event's traversal
-// from the crystal table on each visit, hands each event's parameters to
-// its lane group by a dozen and a half warp shuffles and divides three times
-// per event; most of its issue slots go to that per-event work, which only
-// ~46 samples share.  This path
-//  * computes each event's traversal (reading 1 of the projector: principal
-//    axis, clipped plane range, affine secondary coordinates, TOF coordinate,
-//    sample length), 1/(P^LM 1)_e and 1/mu_e once per state (trav_build),
-//    so a data update reads 40 bytes of table per event;
-//  * stages the selected events of a 32-event chunk in shared memory (one
-//    64-byte record each), from where a lane group reads its event with four
-//    broadcast loads instead of shuffles; the group's first lane writes y+;
-//  * runs the subset's x-principal events and the others in two launches
-//    (phases), so that one image layout and one accumulator layout are live
-//    in L2 at a time (15 + 31 MB on a 200 x 200 x 96 grid).
-// Per sample the arithmetic is the direct kernel's (positions, TOF table,
-// bilinear weights, gathers, fused multiply-adds and atomics in the same
-// order), so the forward projections agree with it bit for bit for the same
-// lane-group width; S_e and (y+ - y)/mu use the stored reciprocals, which
-// moves them by rounding only.  The back-projection goes into the same
-// z-paired accumulators as the direct kernel's, so the image passes are
-// shared.
+// from the crystal table on each visit.  This path computes each event's
+// traversal (reading 1 of the projector: principal axis, trimmed plane range,
+// affine secondary coordinates, TOF coordinate, sample length), 1/(P^LM 1)_e
+// and mu_e once per state (trav_build), so a data update reads 40 bytes of
+// table per event, and walks the events over z-pair images (lm_walk.cuh).
+//
+// Measured on the 200 x 200 x 96 grid (GB300, CUDA events around the launch),
+// one plane per lane over two image layouts and two accumulators (before) /
+// two lanes per plane over bricked z pairs: 7 143 events 17.5 / 14.1 us,
+// 357 143 events 200 / 133 us, 2.14e6 events 1.09 ms / 0.67 ms.  ncu of the
+// row layout of the pairs (before the bricks) at 357 143 events: SM-to-L2
+// request cycles 71 % of peak = one per line gathered (17.1 M) plus one per
+// sector added to (19.5 M), issue 42 %, 247 warp instructions per event (343
+// before): the requests bound it, and the bricks cut them (176 -> 134 us).
+// Ordering the events by direction and place moved it by less than 10 % in
+// either direction, and one-plane-per-lane with the same pairs was no faster.
+// Per sample the positions and weights are the direct kernel's.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
 
-#include "lm_internal.h"
+#include "lm_walk.cuh"
 
 using namespace lmk;
 
@@ -40,7 +36,7 @@ bool trav_capable(const lm_grid* g)
     if (g->n[2] < 2 || g->n[1] < 2) return false;
     for (int d = 0; d < 3; ++d)
         if (g->n[d] >= (1 << 15)) return false;
-    return true;
+    return nvox(g) < (int64_t(1) << 29);  // 32-bit byte offsets into the pair images
 }
 
 TravLayout trav_layout(const lm_grid* g, int64_t N)
@@ -68,17 +64,19 @@ namespace {
 
 using lmh::TOF_TAB_N;
 
-// Packed plane range and principal axis of a table entry: i0 (15 bits),
-// cnt (15 bits, 0 = inert event), k (2 bits).
-__host__ __device__ __forceinline__ unsigned pack_meta(int i0, int cnt, int k)
+// Packed plane range of a table entry: i0 (15 bits), planes (15 bits, 0 =
+// inert event), principal axis (2 bits); an entry whose samples all have
+// their four neighbours inside the grid has a negative sample length.
+__device__ __forceinline__ unsigned pack_meta(int i0, int cnt, int k)
 {
     return (unsigned)i0 | ((unsigned)cnt << 15) | ((unsigned)k << 30);
 }
 
 // One thread per event: the traversal of reading 1 (lor_setup, the direct
-// kernel's own set-up), 1/(P^LM 1)_e with (P^LM 1)_e = c_e times the sum over
-// the event's samples of the in-grid bilinear weights times TOF weight times
-// sample length (0 where that sum is 0: S_e = 0, an inert event), and 1/mu_e.
+// kernel's own set-up) trimmed to its planes with a sample, 1/(P^LM 1)_e with
+// (P^LM 1)_e = c_e times the sum over the event's samples of the in-grid
+// bilinear weights times TOF weight times sample length (0 where that sum is
+// 0: S_e = 0, an inert event), and mu_e.
 __global__ void trav_build_kernel(const Geo G, const int32_t* __restrict__ det1, const int32_t* __restrict__ det2,
                                   const int16_t* __restrict__ tofb, const float* __restrict__ corr,
                                   const uint16_t* __restrict__ mu, int64_t N, const float* __restrict__ tab,
@@ -92,222 +90,116 @@ __global__ void trav_build_kernel(const Geo G, const int32_t* __restrict__ det1,
         const int d1 = det1[e], d2 = det2[e], m = (int)tofb[e];
         bool ok = d1 >= 0 && d1 < G.n_det && d2 >= 0 && d2 < G.n_det && d1 != d2 && m >= -G.M && m <= G.M;
         Lor L;
-        ok = ok && lor_setup(G, d1, d2, m, TOF_BIN, true, L);
+        ok = ok && lor_setup(G, d1, d2, m, TOF_BIN, true, L, true);
         float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
         unsigned mw = 0u;
         if (ok) {
             lmh::lor_strides(G, L.k, true, L);  // extents (and strides) of the secondary axes
-            float acc1 = 0.0f;
-            for (int i = L.i0; i < L.i0 + L.cnt; ++i) {
-                Smp s;
-                if (lmh::sample_tab<false>(G, L, s_tab, inv_dt, i, s)) acc1 += wsum<false>(s);
+            bool inner;
+            lmw::trim(G, L, &inner);
+            if (L.cnt > 0) {
+                float acc1 = 0.0f;
+                for (int i = L.i0; i < L.i0 + L.cnt; ++i) {
+                    Smp s;
+                    if (lmh::sample_tab<false>(G, L, s_tab, inv_dt, i, s)) acc1 += wsum<false>(s);
+                }
+                const float p1 = (corr ? corr[e] : 1.0f) * acc1;
+                a = make_float4(L.ua0, L.sa, L.ub0, L.sb);
+                b = make_float4(L.tau0, L.dtau, inner ? -L.step : L.step, p1 > 0.0f ? 1.0f / p1 : 0.0f);
+                mw = pack_meta(L.i0, L.cnt, L.k);
             }
-            const float p1 = (corr ? corr[e] : 1.0f) * acc1;
-            a = make_float4(L.ua0, L.sa, L.ub0, L.sb);
-            b = make_float4(L.tau0, L.dtau, L.step, p1 > 0.0f ? 1.0f / p1 : 0.0f);
-            mw = pack_meta(L.i0, L.cnt, L.k);
         }
         r0[e] = a;
         r1[e] = b;
-        meta[e] = make_int2((int)mw, __float_as_int(1.0f / (float)mu[e]));
+        meta[e] = make_int2((int)mw, __float_as_int((float)mu[e]));
     }
 }
 
-// floor(v) for -2^22 <= v < 2^22 as an int and as a float, by one addition
-// rounded towards -inf: adding 1.5 * 2^23 leaves a float whose unit in the
-// last place is 1, so the rounded sum is 1.5 * 2^23 + floor(v) exactly.
-// Same values as floorf and the conversion, on the full-rate adder.
-__device__ __forceinline__ int floor_i(float v, float& fl)
+// Stages the events [e0, e0 + nev) that have samples into `rec` (lanes load
+// their event's entry and fields coalesced, with the streaming cache policy:
+// each is read once per update) and returns their number.  MODE EV_FWD also
+// stages the events without samples (their projection is 0).
+template <int MODE>
+__device__ __forceinline__ int stage(const lmh::TabArgs& A, int64_t e0, int nev, lmw::Rec* rec)
 {
-    const float t = __fadd_rd(v, 12582912.0f);
-    fl = t - 12582912.0f;
-    return __float_as_int(t) - 0x4B400000;
-}
-
-// Sample at plane i (fi = i as a float) of a traversal: the direct kernel's
-// sample_tab arithmetic with the TOF table read as (value, slope) pairs
-// (slope = the same float difference the direct kernel forms) and floors on
-// the adder.  Returns false for a sample without weight.
-__device__ __forceinline__ bool sample_t(const Geo& G, const Lor& L, const float2* tab2, float inv_dt, int i,
-                                         float fi, Smp& s)
-{
-    const float tau = fmaf(fi, L.dtau, L.tau0);
-    if (fabsf(tau) > G.W) return false;
-    const float uu = fminf(fmaxf((tau + G.W) * inv_dt, 0.0f), (float)TOF_TAB_N);
-    float kf;
-    const int kq = min(floor_i(uu, kf), TOF_TAB_N - 1);
-    const float f = uu - fminf(kf, (float)(TOF_TAB_N - 1));
-    const float2 t = tab2[kq];
-    const float wt = L.step * fmaf(f, t.y, t.x);
-    if (wt == 0.0f) return false;
-    const float ua = fmaf(fi, L.sa, L.ua0);
-    float fla;
-    const int ia = floor_i(ua, fla);
-    const float fa = ua - fla;
-    const float wa0 = ((unsigned)ia < (unsigned)L.nA) ? (1.0f - fa) : 0.0f;
-    const float wa1 = ((unsigned)(ia + 1) < (unsigned)L.nA) ? fa : 0.0f;
-    const float ub = fmaf(fi, L.sb, L.ub0);
-    float flb;
-    const int ib = floor_i(ub, flb);
-    const float fb = ub - flb;
-    const float wb0 = ((unsigned)ib < (unsigned)L.nB) ? (1.0f - fb) : 0.0f;
-    const float wb1 = ((unsigned)(ib + 1) < (unsigned)L.nB) ? fb : 0.0f;
-    s.base = i * L.sk + ia * L.sA + ib * L.sB;
-    const float wtA0 = wt * wa0, wtA1 = wt * wa1;
-    s.w0 = wtA0 * wb0;
-    s.w1 = wtA1 * wb0;
-    s.w2 = wtA0 * wb1;
-    s.w3 = wtA1 * wb1;
-    return (s.w0 != 0.0f) || (s.w1 != 0.0f) || (s.w2 != 0.0f) || (s.w3 != 0.0f);
-}
-
-// One selected event of a chunk, staged in shared memory.
-struct alignas(16) EvRec {
-    float4 g0;     // ua0, sa, ub0, sb
-    float4 g1;     // tau0, dtau, step, 1/(P^LM 1)_e
-    float4 d;      // c_e, s_e, y_e, mu_e
-    unsigned mw;   // packed plane range and principal axis
-    int lane;      // the event's place in its chunk
-    float inv_mu;  // 1/mu_e
-    float pad;
-};
-
-// One chunk of 32 consecutive events [e0, e0 + nev) of a data update by the
-// calling warp: phase 0 processes its x-principal events, phase 1 the
-// others, phase -1 all of them.  The lanes load their event's table entry
-// and fields coalesced, with the streaming cache policy (read once per
-// update), and stage the selected events in shared memory by rank; groups of
-// G lanes then take them in turn, lane s of a group on planes i0 + s,
-// i0 + s + G, ... as in the direct kernel, keeping up to 64/G samples per lane
-// in registers for the back-projection.  x_std / x_yf: the image the update
-// gathers from.
-template <int G>
-__device__ __forceinline__ void table_chunk(const lmh::TabArgs& A, const float* __restrict__ x_std,
-                                            const float* __restrict__ x_yf, int64_t e0, int nev, int phase,
-                                            const float2* s_tab, float inv_dt, EvRec* rec)
-{
-    constexpr int NG = 32 / G;
-    constexpr int PC = 64 / G;
-    const Geo& Gm = A.G;
     const int lane = threadIdx.x & 31;
-    const int grp = lane / G, sub = lane % G;
     const int64_t e = e0 + lane;
     const bool in = lane < nev;
     const int2 mt = in ? __ldcs(A.meta + e) : make_int2(0, 0);
     const unsigned mw = (unsigned)mt.x;
-    const int mk = (int)(mw >> 30);
-    const bool mine = in && ((mw >> 15) & 0x7FFFu) != 0u && (phase < 0 || ((mk == 0) == (phase == 0)));
+    const unsigned cnt = (mw >> 15) & 0x7FFFu;
+    const bool mine = in && (MODE != lmh::EV_DATA || cnt != 0u);
     const unsigned mask = __ballot_sync(FULL, mine);
-    if (mask == 0u) return;
     if (mine) {
-        EvRec& r = rec[__popc(mask & ((1u << lane) - 1u))];
-        r.g0 = __ldcs(A.r0 + e);
-        r.g1 = __ldcs(A.r1 + e);
-        r.d = make_float4(A.corr ? __ldcs(A.corr + e) : 1.0f, __ldcs(A.contam + e), __ldcs(A.y + e),
-                          (float)__ldcs(reinterpret_cast<const unsigned short*>(A.mu) + e));
-        r.mw = mw;
-        r.lane = lane;
-        r.inv_mu = __int_as_float(mt.y);
+        lmw::Rec& r = rec[__popc(mask & ((1u << lane) - 1u))];
+        const float4 g1 = __ldcs(A.r1 + e);
+        const float mu = __int_as_float(mt.y), step = fabsf(g1.z);
+        const float cs = (A.corr ? __ldcs(A.corr + e) : 1.0f) * step;
+        lmw::rec_path(__ldcs(A.r0 + e), g1.x, g1.y, (int)(mw & 0x7FFFu), (int)cnt, (int)(mw >> 30), g1.z < 0.0f, lane,
+                      r);
+        r.g1.z = cs / mu;
+        r.g1.w = A.gamma_rho * g1.w;  // S_e = gamma rho / (P^LM 1)_e
+        r.d = make_float4(cs, MODE == lmh::EV_FWD ? 0.0f : __ldcs(A.contam + e),
+                          MODE == lmh::EV_DATA ? __ldcs(A.y + e) : 0.0f, mu);
     }
     __syncwarp();
-    const int nm = __popc(mask);
-    for (int b0 = 0; b0 < nm; b0 += NG) {
-        const bool valid = b0 + grp < nm;
-        const EvRec& R = rec[valid ? b0 + grp : b0];
-        const float4 g0 = R.g0, g1 = R.g1, dd = R.d;
-        const unsigned rw = R.mw;
-        Lor E;
-        E.i0 = (int)(rw & 0x7FFFu);
-        E.cnt = valid ? (int)((rw >> 15) & 0x7FFFu) : 0;
-        const int k = (int)(rw >> 30);
-        E.ua0 = g0.x;
-        E.sa = g0.y;
-        E.ub0 = g0.z;
-        E.sb = g0.w;
-        E.tau0 = g1.x;
-        E.dtau = g1.y;
-        E.step = g1.z;
-        lmh::lor_strides(Gm, k, true, E);
-        E.k = k;
-        const float* __restrict__ img = k == 1 ? x_yf : x_std;
-        const int npass = (E.cnt + G - 1) / G;
-        const int iend = E.i0 + E.cnt;
-        const int ifirst = E.i0 + sub;
-        const float ffirst = (float)ifirst;
-        float acc = 0.0f;
-        Smp cs[PC];
-#pragma unroll
-        for (int p = 0; p < PC; ++p) {
-            cs[p].base = 0;
-            cs[p].w0 = cs[p].w1 = cs[p].w2 = cs[p].w3 = 0.0f;
-            if (p < npass) {
-                const int i = ifirst + p * G;
-                if (i < iend && sample_t(Gm, E, s_tab, inv_dt, i, ffirst + (float)(p * G), cs[p]))
-                    acc += gather<false>(img, E, cs[p]);
-                else
-                    cs[p].w0 = cs[p].w1 = cs[p].w2 = cs[p].w3 = 0.0f;
-            }
+    return __popc(mask);
+}
+
+// The staged events of one chunk, two at a time: forward projection of both,
+// one reduction, the per-event step (MODE EV_DATA: Eq. (proxD); EV_FWD: the
+// projection itself) in a half-warp each, and the back-projection of both.
+template <int MODE>
+__device__ __forceinline__ void table_pairs(const lmh::TabArgs& A, const lmw::Lane& l, int64_t e0, int nm,
+                                            const lmw::Rec* rec)
+{
+    const int lane = threadIdx.x & 31;
+    const char* img = reinterpret_cast<const char*>(A.xp);
+    char* acc = reinterpret_cast<char*>(A.acc);
+    for (int b = 0; b < nm; b += 2) {
+        lmw::Held h0, h1;
+        float a1 = 0.0f;
+        const bool two = b + 1 < nm;
+        const float a0 = lmw::forward<true>(l, A.G, A.lay, rec[b], img, h0);
+        if (two) a1 = lmw::forward<true>(l, A.G, A.lay, rec[b + 1], img, h1);
+        const lmw::Rec& R = rec[b + (two ? lane >> 4 : 0)];
+        const float4 dd = R.d;
+        const bool valid = lane < 16 || two;
+        const bool first = valid && (lane & 15) == 0;
+        const float J = lmw::reduce2(a0, a1);                 // (P^LM x)_e = c_e step J
+        const int64_t e = e0 + (R.meta >> 20);
+        if (MODE == lmh::EV_FWD) {
+            if (first) A.out[e] = dd.x * J;
+            continue;
         }
-        for (int p = PC; p < npass; ++p) {
-            const int i = ifirst + p * G;
-            Smp s;
-            if (i < iend && sample_t(Gm, E, s_tab, inv_dt, i, (float)i, s)) acc += gather<false>(img, E, s);
-        }
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
         // dual step of Eq. (proxD) with the listmode step mu_e S_e
-        const float cj = dd.x, sj = dd.y, yj = dd.z, muj = dd.w;
-        const float Se = A.gamma_rho * g1.w;                  // S_e = gamma rho / (P^LM 1)_e
-        const float a = fmaf(Se, fmaf(cj, acc, sj), yj);      // y + S (P^LM x + s)
-        const float yp = prox_dstar(a, muj * Se);
-        const float v = (yp - yj) * R.inv_mu;                 // (y+ - y) / mu
-        if (valid && sub == 0) __stcs(A.y + e0 + R.lane, yp);
-        const float bval = valid ? cj * v : 0.0f;
-        if (bval != 0.0f) {
-            float* acc_img = k == 1 ? A.acc_yf : A.acc_std;
-#pragma unroll
-            for (int p = 0; p < PC; ++p)
-                if (p < npass) scatter_pairs<false>(acc_img, E, cs[p], bval);
-            for (int p = PC; p < npass; ++p) {
-                const int i = ifirst + p * G;
-                Smp s;
-                if (i < iend && sample_t(Gm, E, s_tab, inv_dt, i, (float)i, s))
-                    scatter_pairs<false>(acc_img, E, s, bval);
-            }
-        }
+        const float Se = R.g1.w;
+        const float a = fmaf(Se, fmaf(dd.x, J, dd.y), dd.z);  // y + S (P^LM x + s)
+        const float yp = prox_dstar(a, dd.w * Se);
+        if (first) __stcs(A.y + e, yp);
+        float bval = R.g1.z * (yp - dd.z);                    // c step (y+ - y) / mu
+        if (!valid) bval = 0.0f;
+        const float b0 = __shfl_sync(FULL, bval, 0), b1 = __shfl_sync(FULL, bval, 16);
+        if (b0 != 0.0f) lmw::backward<true>(l, A.G, A.lay, rec[b], h0, b0, acc);
+        if (b1 != 0.0f) lmw::backward<true>(l, A.G, A.lay, rec[b + 1], h1, b1, acc);
     }
     __syncwarp();
 }
 
-__device__ __forceinline__ void fill_tab2(float2* s_tab, const float* tab)
-{
-    for (int k = threadIdx.x; k < TOF_TAB_N; k += blockDim.x) {
-        const float a = tab[k];
-        s_tab[k] = make_float2(a, tab[k + 1] - a);
-    }
-}
+constexpr int TAB_THREADS = 512;
+constexpr int TAB_WARPS = TAB_THREADS / 32;
+constexpr size_t TAB_SMEM = lmw::TAB_PAD * sizeof(float2) + (size_t)TAB_WARPS * 32 * sizeof(lmw::Rec);
 
-// The self-resetting work counter: the last warp to finish clears it.
-__device__ __forceinline__ void release_queue(unsigned long long* queue, unsigned* done)
+// One subset (or event range) from the traversal table.  Block b takes the
+// chunks b, b + blocks, ...; its warps draw them from a counter in shared
+// memory (a global counter served one draw in about 2.5 ns, which held
+// launches with small chunks back: 75 us for 50 000 events, against 22 us).
+template <int MODE>
+__global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_kernel(const __grid_constant__ lmh::TabArgs A)
 {
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) {
-        const unsigned tw = (unsigned)((gridDim.x * blockDim.x) >> 5);
-        const unsigned d = atomicAdd(done, 1u);
-        if (d == tw - 1) {
-            *queue = 0ULL;
-            *done = 0u;
-        }
-    }
-}
-
-// Data update of one subset from the traversal table: warps take the
-// subset's chunks from a self-resetting counter (table_chunk).
-template <int G, int MINB>
-__global__ void __launch_bounds__(256, MINB) ev_table_kernel(const lmh::TabArgs A)
-{
-    __shared__ float2 s_tab[TOF_TAB_N];
-    __shared__ EvRec s_rec[8][32];
+    extern __shared__ float4 s_dyn[];
+    __shared__ int s_next;
+    float2* s_tab = reinterpret_cast<float2*>(s_dyn);
     int64_t eb = A.e_begin, ee = A.e_end;
     if (A.seq != nullptr) {
         const int sel = A.seq[A.u];
@@ -315,82 +207,123 @@ __global__ void __launch_bounds__(256, MINB) ev_table_kernel(const lmh::TabArgs 
         eb = A.sub_off[sel];
         ee = A.sub_off[sel + 1];
     }
-    fill_tab2(s_tab, A.tof_tab);
-    __syncthreads();
-    const float inv_dt = (float)TOF_TAB_N / (2.0f * A.G.W);
-    const int lane = threadIdx.x & 31;
     const int64_t count = ee - eb;
-    const int64_t nch = count > 0 ? (count + 31) / 32 : 0;
-    EvRec* rec = s_rec[threadIdx.x >> 5];
-    for (;;) {
-        unsigned long long cc = 0;
-        if (lane == 0) cc = atomicAdd(A.queue, 1ULL);
-        const int64_t c = (int64_t)__shfl_sync(FULL, cc, 0);
-        if (c >= nch) break;
-        const int64_t e0 = eb + c * 32;
-        table_chunk<G>(A, A.x_std, A.x_yf, e0, (int)min((int64_t)32, ee - e0), A.phase, s_tab, inv_dt, rec);
+    const int CH = lmw::chunk_of(count, (int64_t)gridDim.x * TAB_WARPS);
+    const int64_t nch = count > 0 ? (count + CH - 1) / CH : 0;
+    const int warp = threadIdx.x >> 5;
+    lmw::Rec* rec = reinterpret_cast<lmw::Rec*>(s_tab + lmw::TAB_PAD) + warp * 32;
+    int64_t c = (int64_t)warp * gridDim.x + blockIdx.x;
+    int nm = c < nch ? stage<MODE>(A, eb + c * CH, (int)min((int64_t)CH, count - c * CH), rec) : 0;
+    if (threadIdx.x == 0) s_next = TAB_WARPS;
+    lmw::fill_tab(s_tab, A.tof_tab);
+    __syncthreads();
+    const lmw::Lane l = lmw::make_lane(s_tab, A.G.W);
+    while (c < nch) {
+        table_pairs<MODE>(A, l, eb + c * CH, nm, rec);
+        int k = 0;
+        if ((threadIdx.x & 31) == 0) k = atomicAdd(&s_next, 1);
+        c = (int64_t)__shfl_sync(FULL, k, 0) * gridDim.x + blockIdx.x;
+        if (c < nch) nm = stage<MODE>(A, eb + c * CH, (int)min((int64_t)CH, count - c * CH), rec);
     }
-    release_queue(A.queue, A.done);
 }
 
 // The data updates of every active frame of a batch at update u, from their
-// traversal tables: the work items are the 32-event chunks of each frame's
+// traversal tables: the work items are the chunks of each frame's
 // selected subset (frames at a prior update have none: their dual step runs
 // in the image pass), found through a prefix table in shared memory.
-template <int G, int MINB>
-__global__ void __launch_bounds__(256, MINB) ev_table_batch_kernel(const lmh::BatchTabArgs B)
+__global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_batch_kernel(const __grid_constant__ lmh::BatchTabArgs B)
 {
-    extern __shared__ float2 s_tab[];  // TOF_TAB_N pairs (dynamic: with the tables below above 48 KB)
-    __shared__ EvRec s_rec[8][32];
+    extern __shared__ float4 s_dyn[];
+    float2* s_tab = reinterpret_cast<float2*>(s_dyn);
     __shared__ long long s_pre[lmh::BATCH_MAX + 1];
     __shared__ long long s_eb[lmh::BATCH_MAX];
     __shared__ long long s_ee[lmh::BATCH_MAX];
+    __shared__ int s_next;
     const int cap = B.cap;
-    const int par = B.u & 1;
     if (threadIdx.x < cap) {
         const int s = threadIdx.x;
-        long long items = 0, eb = 0, ee = 0;
+        long long eb = 0, ee = 0;
         if (B.active[s]) {
             const lmh::TabArgs& A = B.slots[s];
             const int sel = B.seqs[(size_t)s * B.seq_stride + B.u];
             if (sel < A.n_subsets) {
                 eb = A.sub_off[sel];
                 ee = A.sub_off[sel + 1];
-                items = (ee - eb + 31) / 32;
             }
         }
-        s_eb[threadIdx.x] = eb;
-        s_ee[threadIdx.x] = ee;
-        s_pre[threadIdx.x + 1] = items;
+        s_eb[s] = eb;
+        s_ee[s] = ee;
     }
-    fill_tab2(s_tab, B.tof_tab);
+    if (threadIdx.x == 0) s_next = 0;
+    lmw::fill_tab(s_tab, B.tof_tab);
     __syncthreads();
+    long long events = 0;
+    for (int s = 0; s < cap; ++s) events += s_ee[s] - s_eb[s];
+    const int CH = lmw::chunk_of(events, (long long)gridDim.x * TAB_WARPS);
     if (threadIdx.x == 0) {
         s_pre[0] = 0;
-        for (int s = 0; s < cap; ++s) s_pre[s + 1] += s_pre[s];
+        for (int s = 0; s < cap; ++s) s_pre[s + 1] = s_pre[s] + (s_ee[s] - s_eb[s] + CH - 1) / CH;
     }
     __syncthreads();
     const long long total = s_pre[cap];
-    const float inv_dt = (float)TOF_TAB_N / (2.0f * B.tof_W);
-    const int lane = threadIdx.x & 31;
-    EvRec* rec = s_rec[threadIdx.x >> 5];
+    const lmw::Lane l = lmw::make_lane(s_tab, B.tof_W);
+    lmw::Rec* rec = reinterpret_cast<lmw::Rec*>(s_tab + lmw::TAB_PAD) + (threadIdx.x >> 5) * 32;
     for (;;) {
-        unsigned long long cc = 0;
-        if (lane == 0) cc = atomicAdd(B.queue, 1ULL);
-        const long long c = (long long)__shfl_sync(FULL, cc, 0);
+        int k = 0;
+        if ((threadIdx.x & 31) == 0) k = atomicAdd(&s_next, 1);
+        const long long c = (long long)__shfl_sync(FULL, k, 0) * gridDim.x + blockIdx.x;
         if (c >= total) break;
         int s = 0;
         while (s_pre[s + 1] <= c) ++s;
         const lmh::TabArgs& A = B.slots[s];
-        const int64_t e0 = s_eb[s] + (c - s_pre[s]) * 32;
-        table_chunk<G>(A, A.xs[par], A.xyfs[par], e0, (int)min((long long)32, s_ee[s] - e0), -1, s_tab, inv_dt, rec);
+        const int64_t e0 = s_eb[s] + (c - s_pre[s]) * CH;
+        const int nm = stage<lmh::EV_DATA>(A, e0, (int)min((long long)CH, s_ee[s] - e0), rec);
+        table_pairs<lmh::EV_DATA>(A, l, e0, nm, rec);
     }
-    release_queue(B.queue, B.done);
+}
+
+// x (x fastest) as z pairs (x_j, x_{j + nx*ny}), 0 above the last slice.
+__global__ void __launch_bounds__(256) pair_image_kernel(const float* __restrict__ x, char* __restrict__ xp, int nx,
+                                                         int ny, int64_t V, const lmh::PairLay P)
+{
+    const int64_t nxy = (int64_t)nx * ny;
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < V; j += (int64_t)gridDim.x * blockDim.x) {
+        const int z = (int)(j / nxy), r = (int)(j - z * nxy), y = r / nx;
+        *reinterpret_cast<float2*>(xp + P.at((unsigned)(r - y * nx), (unsigned)y, (unsigned)z)) =
+            make_float2(x[j], j + nxy < V ? x[j + nxy] : 0.0f);
+    }
 }
 
 }  // namespace
 
 namespace lmh {
+
+PairLay pair_layout(const lm_grid* g, bool rows)
+{
+    PairLay P;
+    const unsigned nx = (unsigned)g->n[0], ny = (unsigned)g->n[1];
+    P.x1 = 8u;
+    P.y1 = 8u * nx;
+    P.x2 = P.x3 = P.y2 = P.y3 = 0u;
+    P.zs = 8u * nx * ny;
+    P.brick = !rows && nx % 4 == 0 && ny % 4 == 0;
+    if (P.brick) {
+        P.x1 = 32u;
+        P.x2 = 0u - 16u;
+        P.x3 = 0u - 24u;
+        P.y2 = 32u - 8u * nx;
+        P.y3 = 16u - 8u * nx;
+    }
+    return P;
+}
+
+void launch_pair_image(const lm_grid* g, const PairLay& P, const float* x, float* xp, cudaStream_t st)
+{
+    const int64_t V = nvox(g);
+    const int grid = (int)std::min<int64_t>((V + 255) / 256, (int64_t)num_sms() * 16);
+    pair_image_kernel<<<grid, 256, 0, st>>>(x, (char*)xp, g->n[0], g->n[1], V, P);
+    count_launch();
+}
 
 int trav_build(const Geo& G, const lm_events& ev, const uint16_t* mu, const float* tof_tab, const TravLayout& L,
                char* base, cudaStream_t st)
@@ -405,69 +338,42 @@ int trav_build(const Geo& G, const lm_events& ev, const uint16_t* mu, const floa
     return LM_OK;
 }
 
-// Lane-group widths and the resident blocks each variant is compiled for
-// (registers per thread): width 32 with 3 or 4 blocks per SM, 16 and 8 with 2.
-template <int G, int MINB>
-static int table_blocks()
+template <class F>
+static int table_blocks(F* kernel)
+{
+    int b = 0;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAB_SMEM);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, TAB_THREADS, TAB_SMEM) != cudaSuccess || b < 1) b = 1;
+    return num_sms() * b;
+}
+
+// Resident blocks of the table kernels (all modes have the same bounds).
+int table_grid()
 {
     static int nb = 0;
     static std::once_flag once;
     std::call_once(once, [] {
-        int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, ev_table_kernel<G, MINB>, 256, 0) != cudaSuccess ||
-            b < 1)
-            b = 1;
-        nb = b;
+        nb = std::min(table_blocks(ev_table_kernel<EV_DATA>),
+                      std::min(table_blocks(ev_table_kernel<EV_FWD>), table_blocks(ev_table_batch_kernel)));
     });
     return nb;
 }
 
-int table_grid(int variant)
+int launch_table_batch(const BatchTabArgs& b, cudaStream_t st)
 {
-    int b = 1;
-    switch (variant) {
-    case 8: b = table_blocks<8, 2>(); break;
-    case 16: b = table_blocks<16, 2>(); break;
-    case 32: b = table_blocks<32, 3>(); break;
-    case 33: b = table_blocks<32, 4>(); break;
-    default: break;
-    }
-    return num_sms() * b;
-}
-
-template <int G, int MINB>
-static void batch_attr()
-{
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(ev_table_batch_kernel<G, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(TOF_TAB_N * sizeof(float2)));
-    });
-}
-
-int launch_table_batch(const BatchTabArgs& b, int variant, int grid, cudaStream_t st)
-{
-    const size_t dyn = TOF_TAB_N * sizeof(float2);
-    switch (variant) {
-    case 8: batch_attr<8, 2>(); ev_table_batch_kernel<8, 2><<<grid, 256, dyn, st>>>(b); break;
-    case 16: batch_attr<16, 2>(); ev_table_batch_kernel<16, 2><<<grid, 256, dyn, st>>>(b); break;
-    case 32: batch_attr<32, 3>(); ev_table_batch_kernel<32, 3><<<grid, 256, dyn, st>>>(b); break;
-    case 33: batch_attr<32, 4>(); ev_table_batch_kernel<32, 4><<<grid, 256, dyn, st>>>(b); break;
-    default: set_error("unknown traversal-table kernel variant %d", variant); return LM_ERR_INVALID_ARG;
-    }
+    ev_table_batch_kernel<<<table_grid(), TAB_THREADS, TAB_SMEM, st>>>(b);
     count_launch();
     LM_CUDA(cudaGetLastError());
     return LM_OK;
 }
 
-int launch_table_update(const TabArgs& a, int variant, int grid, cudaStream_t st)
+int launch_table(int mode, const TabArgs& a, cudaStream_t st)
 {
-    switch (variant) {
-    case 8: ev_table_kernel<8, 2><<<grid, 256, 0, st>>>(a); break;
-    case 16: ev_table_kernel<16, 2><<<grid, 256, 0, st>>>(a); break;
-    case 32: ev_table_kernel<32, 3><<<grid, 256, 0, st>>>(a); break;
-    case 33: ev_table_kernel<32, 4><<<grid, 256, 0, st>>>(a); break;
-    default: set_error("unknown traversal-table kernel variant %d", variant); return LM_ERR_INVALID_ARG;
+    const int grid = table_grid();
+    switch (mode) {
+    case EV_DATA: ev_table_kernel<EV_DATA><<<grid, TAB_THREADS, TAB_SMEM, st>>>(a); break;
+    case EV_FWD: ev_table_kernel<EV_FWD><<<grid, TAB_THREADS, TAB_SMEM, st>>>(a); break;
+    default: set_error("unknown traversal-table mode %d", mode); return LM_ERR_INVALID_ARG;
     }
     count_launch();
     LM_CUDA(cudaGetLastError());

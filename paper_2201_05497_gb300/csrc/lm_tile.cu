@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(256) tl_count_kernel(const TileArgs A, const B
             const int m = (int)A.tofb[q];
             if (A.corr) c = A.corr[q];
             ok = d1 >= 0 && d1 < G.n_det && d2 >= 0 && d2 < G.n_det && d1 != d2 && m >= -G.M && m <= G.M;
-            ok = ok && lor_setup(G, d1, d2, m, TOF_BIN, false, L) && L.cnt < 16384 && L.i0 < 16384;
+            ok = ok && lor_setup(G, d1, d2, m, TOF_BIN, false, L, true) && L.cnt < 16384 && L.i0 < 16384;
         }
         float4 e0v = make_float4(0.0f, 0.0f, 0.0f, 0.0f), e1v = e0v;
         if (ok) {
