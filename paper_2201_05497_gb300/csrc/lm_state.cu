@@ -912,8 +912,9 @@ int lmspdhg_create(lm_state** out, const lm_scanner* sc, const lm_grid* grid, co
     }
     st->table = false;
     st->tv_base = nullptr;
+    // (the pair images are addressed by 32-bit byte offsets; larger grids keep the direct kernel)
     if (P.trav_buf != nullptr && tof->n_bins > 0 && !st->det && !st->has_res && !P.sinogram && !st->tiled &&
-        trav_capable(grid)) {
+        trav_capable(grid) && st->V < (int64_t(1) << 29)) {
         st->tv = trav_layout(grid, ev->n);
         char* tb = (char*)(((uintptr_t)P.trav_buf + 255) / 256 * 256);
         if (P.trav_bytes < st->tv.total || P.trav_bytes - (size_t)(tb - (char*)P.trav_buf) < st->tv.total - 256) {

@@ -36,7 +36,7 @@ bool trav_capable(const lm_grid* g)
     if (g->n[2] < 2 || g->n[1] < 2) return false;
     for (int d = 0; d < 3; ++d)
         if (g->n[d] >= (1 << 15)) return false;
-    return nvox(g) < (int64_t(1) << 29);  // 32-bit byte offsets into the pair images
+    return true;
 }
 
 TravLayout trav_layout(const lm_grid* g, int64_t N)

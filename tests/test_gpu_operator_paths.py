@@ -1,0 +1,46 @@
+"""GPU: the standalone operators where their launch rules branch: projections
+of many events (TOF weights from a table per block) against the same events
+in small calls (an erf per sample)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2201_05497_gb300 import synth as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lm():
+    from paper_2201_05497_gb300 import build, lm as _lm
+    build.build()
+    _lm.load_library()
+    return _lm
+
+
+@pytest.mark.parametrize("two_d", [False, True])
+def test_many_events_equal_few(lm, two_d):
+    """The table interpolates the TOF kernel to 1e-7 of its peak and erf
+    carries as much, so a projection moves by at most 4e-7 of the largest."""
+    sc = S.Scanner(1, 128, 150.0, 1.0) if two_d else S.Scanner(8, 96, 150.0, 8.0)
+    g = S.Grid((41, 37, 1 if two_d else 14), (5.0, 5.0, 5.0))
+    tof = S.tof_400ps(27, 600.0 / 27)
+    n = 90000
+    ev = S.uniform_events(sc, tof, n, 5)
+    geo = lm.Geometry(torch.from_numpy(sc.crystal_table()).cuda(), sc.n_rings, sc.n_xtal, g.n, g.h, g.origin, tof.sigma,
+                      tof.bin, tof.n_sigma, tof.n_bins)
+    dev = lm.DeviceEvents.from_numpy(ev)
+    rng = np.random.default_rng(2)
+    x = torch.from_numpy(rng.uniform(0.1, 1, geo.V).astype(np.float32)).cuda()
+    v = torch.from_numpy(rng.normal(size=n).astype(np.float32)).cuda()
+    p = lm.fwd(geo, x, dev).double()
+    b = lm.back(geo, v, dev).double()
+    ps, bs = [], torch.zeros(geo.V, dtype=torch.float64, device="cuda")
+    for s in range(0, n, 6000):
+        part = lm.DeviceEvents(*[t[s:s + 6000].contiguous() for t in (dev.det1, dev.det2, dev.tof, dev.corr, dev.contam)])
+        ps.append(lm.fwd(geo, x, part).double())
+        bs += lm.back(geo, v[s:s + 6000].contiguous(), part).double()
+    ps = torch.cat(ps)
+    assert float((p - ps).abs().max()) <= 4e-7 * float(ps.abs().max()) * 4  # four taps
+    assert float((b - bs).norm() / bs.norm()) <= 2e-6
