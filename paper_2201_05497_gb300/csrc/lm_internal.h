@@ -369,6 +369,24 @@ struct BatchTabArgs {
 int launch_table_batch(const BatchTabArgs& b, cudaStream_t st);
 int trav_build(const lmk::Geo& G, const lm_events& ev, const uint16_t* mu, const float* tof_tab,
                const TravLayout& L, char* base, cudaStream_t st);
+// Standalone projections by the table projector's walk: EV_FWD out[e] = c_e J_e x
+// from xp, EV_BACK acc += c_e v_e J_e^T.
+struct OpArgs {
+    lmk::Geo G;
+    PairLay lay;
+    const int32_t* det1;
+    const int32_t* det2;
+    const int16_t* tof;
+    const float* corr;
+    const float* v;
+    int64_t n;
+    const float* xp;
+    float* out;
+    float* acc;
+};
+int launch_op(int mode, const OpArgs& a, cudaStream_t st);
+// img += the pair accumulator
+void launch_pair_fold(const lm_grid* g, const PairLay& P, float* img, const float* acc, cudaStream_t st);
 // xp = x as z pairs (voxel j, voxel j + nx*ny)
 void launch_pair_image(const lm_grid* g, const PairLay& P, const float* x, float* xp, cudaStream_t st);
 // mode: EV_DATA or EV_FWD (out[e] = c_e J_e x)

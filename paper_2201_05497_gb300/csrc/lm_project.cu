@@ -1220,6 +1220,37 @@ static int operator_shape(EvArgs& a, int mode, bool two_d)
     return grid;
 }
 
+// The table projector's walk serves the standalone projections of 3D grids
+// from WALK_EVENTS on, where its pair image (8 bytes per voxel of workspace)
+// and the table each block makes are repaid; fewer events, 2D grids, smaller
+// workspaces (4 bytes per voxel served before) and 2^29 voxels or more take the
+// event kernel.
+constexpr int64_t WALK_EVENTS = 16384;
+
+static bool walk_grid(const lm_grid* g) { return trav_capable(g) && nvox(g) < (int64_t(1) << 29); }
+
+static size_t op_workspace(const lm_grid* g) { return align_up((size_t)nvox(g) * (walk_grid(g) ? 8 : 4)); }
+
+static bool use_walk(const lm_grid* g, int64_t n, const void* ws, size_t ws_bytes)
+{
+    return walk_grid(g) && n >= WALK_EVENTS && ws != nullptr && ws_bytes >= op_workspace(g) &&
+           ((uintptr_t)ws & 15) == 0;
+}
+
+static OpArgs op_args(const lmk::Geo& G, const lm_grid* g, const lm_events* ev)
+{
+    OpArgs o;
+    std::memset(&o, 0, sizeof(o));
+    o.G = G;
+    o.lay = pair_layout(g, false);
+    o.det1 = ev->det1;
+    o.det2 = ev->det2;
+    o.tof = ev->tof;
+    o.corr = ev->corr;
+    o.n = ev->n;
+    return o;
+}
+
 static float step_max(const lm_grid* g)
 {
     return 2.0f * std::fmax(g->h[0], std::fmax(g->h[1], g->h[2]));
@@ -1252,7 +1283,7 @@ int64_t lm_n_lor(const lm_scanner* sc)
 size_t lm_fwd_workspace_bytes(const lm_grid* grid)
 {
     if (check_grid(grid)) return 0;
-    return align_up((size_t)nvox(grid) * 4);
+    return op_workspace(grid);
 }
 
 int lm_fwd(const lm_scanner* sc, const lm_grid* grid, const lm_tof* tof, const float* x, const lm_events* ev,
@@ -1268,11 +1299,18 @@ int lm_fwd(const lm_scanner* sc, const lm_grid* grid, const lm_tof* tof, const f
     LM_CHECK(x != nullptr && p != nullptr, LM_ERR_INVALID_ARG, "x or p is NULL");
     LM_CHECK(tof->n_bins == 0 || ev->tof != nullptr, LM_ERR_INVALID_ARG, "TOF bins NULL for a TOF scanner");
     cudaStream_t st = S(stream);
+    if (use_walk(grid, ev->n, ws, ws_bytes)) {
+        OpArgs o = op_args(G, grid, ev);
+        launch_pair_image(grid, o.lay, x, (float*)ws, st);
+        o.xp = (const float*)ws;
+        o.out = p;
+        return launch_op(EV_FWD, o, st);
+    }
     EvArgs a;
     std::memset(&a, 0, sizeof(a));
     a.G = G;
     a.x_std = x;
-    if (ws != nullptr && ws_bytes >= lm_fwd_workspace_bytes(grid) && grid->n[1] > 1) {
+    if (ws != nullptr && ws_bytes >= align_up((size_t)nvox(grid) * 4) && grid->n[1] > 1) {
         launch_transpose_to_yf(grid, x, (float*)ws, st);
         a.x_yf = (const float*)ws;
     }
@@ -1296,7 +1334,7 @@ size_t lm_back_workspace_bytes(const lm_grid* grid, int deterministic)
     if (check_grid(grid)) return 0;
     const size_t V = (size_t)nvox(grid);
     if (deterministic) return 2 * align_up(V * 8) + 256;
-    return align_up(V * 4);
+    return op_workspace(grid);
 }
 
 int lm_back(const lm_scanner* sc, const lm_grid* grid, const lm_tof* tof, const lm_events* ev, const float* v,
@@ -1311,13 +1349,25 @@ int lm_back(const lm_scanner* sc, const lm_grid* grid, const lm_tof* tof, const 
     if (ev->n == 0) return LM_OK;
     LM_CHECK(v != nullptr && img != nullptr, LM_ERR_INVALID_ARG, "v or img is NULL");
     LM_CHECK(tof->n_bins == 0 || ev->tof != nullptr, LM_ERR_INVALID_ARG, "TOF bins NULL for a TOF scanner");
-    const size_t need = lm_back_workspace_bytes(grid, deterministic);
+    // (float mode: the y-fastest copy; the walk takes twice that where there is room)
+    const size_t need = deterministic ? lm_back_workspace_bytes(grid, 1) : align_up((size_t)nvox(grid) * 4);
     LM_CHECK(!deterministic || (ws != nullptr && ws_bytes >= need), LM_ERR_NOMEM,
              "deterministic back-projection needs %zu workspace bytes", need);
     cudaStream_t st = S(stream);
     const size_t V = (size_t)nvox(grid);
     const bool two_d = grid->n[2] == 1 && sc->n_rings == 1;  // single-ring scanner in the image plane
     const bool use_yf = grid->n[1] > 1 && ws != nullptr && ws_bytes >= need;
+    if (!deterministic && use_walk(grid, ev->n, ws, ws_bytes)) {
+        OpArgs o = op_args(G, grid, ev);
+        o.v = v;
+        o.acc = (float*)ws;
+        LM_CUDA(cudaMemsetAsync(ws, 0, V * 8, st));
+        rc = launch_op(EV_BACK, o, st);
+        if (rc) return rc;
+        launch_pair_fold(grid, o.lay, img, (const float*)ws, st);
+        LM_CUDA(cudaGetLastError());
+        return LM_OK;
+    }
     EvArgs a;
     std::memset(&a, 0, sizeof(a));
     a.G = G;

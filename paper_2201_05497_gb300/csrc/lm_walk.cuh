@@ -64,6 +64,24 @@ __device__ __forceinline__ void fill_tab(float2* s_tab, const float* __restrict_
     }
 }
 
+// The same table made by the block itself.  The kernel is even; erfc keeps
+// the relative accuracy of its tails.  Ends with a barrier.
+__device__ __forceinline__ void make_tab(float2* s_tab, const Geo& G)
+{
+    const float hb = 0.5f * G.bin, dt = 2.0f * G.W / (float)TOF_TAB_N;
+    for (int k = threadIdx.x; k <= TOF_TAB_N / 2; k += blockDim.x) {
+        const float tau = G.W - dt * (float)k;
+        const float w = 0.5f * (erfcf((tau - hb) * G.inv_s) - erfcf((tau + hb) * G.inv_s));
+        s_tab[k + 1].x = w;
+        s_tab[TOF_TAB_N - k + 1].x = w;
+        if (k == 0) s_tab[0].x = w;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < TAB_PAD; k += blockDim.x)
+        s_tab[k].y = k == 0 || k == TAB_PAD - 1 ? 0.0f : s_tab[k + 1].x - s_tab[k].x;
+    __syncthreads();
+}
+
 // Trims the plane range of a traversal (lor_setup widens it by a plane on
 // each side) to the planes with a sample: |tau| <= W and a neighbour inside
 // the grid.  The coordinates are monotone in the plane, so these planes are
@@ -164,8 +182,9 @@ __device__ __forceinline__ unsigned along(const AxisLay& a, unsigned i)
 // (which keeps the table index in range) without a sample.  INNER: all
 // neighbours are inside the grid; otherwise a neighbour outside weighs 0, and
 // a sample whose slice B is below the grid takes the first half of slice 0.
+// SAFE: a voxel of weight 0 does not enter (it may hold an infinity or NaN).
 // Returns the lane's part of sum w x / (c_e step).
-template <int NP, int CHECK, bool INNER, bool TOF, bool GATHER>
+template <int NP, int CHECK, bool INNER, bool TOF, bool GATHER, bool SAFE>
 __device__ __forceinline__ float walk(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r, int p0,
                                       const char* __restrict__ img, Held& h)
 {
@@ -218,6 +237,10 @@ __device__ __forceinline__ float walk(const Lane& l, const Geo& G, const lmh::Pa
         if (GATHER) {
             x[p] = make_float2(0.0f, 0.0f);
             if ((INNER && p < CHECK) || off != NONE) x[p] = __ldg(reinterpret_cast<const float2*>(img + off));
+            if (SAFE) {
+                if (q0 == 0.0f) x[p].x = 0.0f;
+                if (q1 == 0.0f) x[p].y = 0.0f;
+            }
         }
     }
     float acc = 0.0f;
@@ -265,7 +288,7 @@ __device__ __noinline__ float walk_z(const Lane l, const Geo& G, const lmh::Pair
 
 // Forward part of one event.  Planes beyond the held ones (finer grids) are
 // walked sixteen at a time.
-template <bool TOF>
+template <bool TOF, bool SAFE = false>
 __device__ __forceinline__ float forward(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r,
                                          const char* __restrict__ img, Held& h)
 {
@@ -275,14 +298,14 @@ __device__ __forceinline__ float forward(const Lane& l, const Geo& G, const lmh:
     if (((m >> 15) & 3u) == 2u) return walk_z<TOF>(l, G, P, r, img, nullptr, false, 0.0f);
     float acc;
     if ((m & REC_INNER) && cnt > 32) {
-        if (cnt > 48) acc = walk<4, 3, true, TOF, true>(l, G, P, r, 0, img, h);
-        else acc = walk<3, 2, true, TOF, true>(l, G, P, r, 0, img, h);
+        if (cnt > 48) acc = walk<4, 3, true, TOF, true, SAFE>(l, G, P, r, 0, img, h);
+        else acc = walk<3, 2, true, TOF, true, SAFE>(l, G, P, r, 0, img, h);
     } else {
-        acc = walk<4, 0, false, TOF, true>(l, G, P, r, 0, img, h);
+        acc = walk<4, 0, false, TOF, true, SAFE>(l, G, P, r, 0, img, h);
     }
     for (int p = PASSES; 16 * p < cnt; ++p) {
         Held t;
-        acc += walk<1, 0, false, TOF, true>(l, G, P, r, p, img, t);
+        acc += walk<1, 0, false, TOF, true, SAFE>(l, G, P, r, p, img, t);
     }
     return acc;
 }
@@ -304,10 +327,27 @@ __device__ __forceinline__ void backward(const Lane& l, const Geo& G, const lmh:
             atomicAdd(reinterpret_cast<float2*>(acc + h.off[p]), make_float2(h.q0[p] * b, h.q1[p] * b));
     for (int p = PASSES; 16 * p < cnt; ++p) {
         Held t;
-        walk<1, 0, false, TOF, false>(l, G, P, r, p, nullptr, t);
+        walk<1, 0, false, TOF, false, false>(l, G, P, r, p, nullptr, t);
         if (t.off[0] != NONE)
             atomicAdd(reinterpret_cast<float2*>(acc + t.off[0]), make_float2(t.q0[0] * b, t.q1[0] * b));
     }
+}
+
+// Back-projection of one event that was not walked forward before.
+template <bool TOF>
+__device__ __forceinline__ void spread(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r, float b, char* acc)
+{
+    const unsigned m = r.meta;
+    const int cnt = (int)(m & 0x7FFFu);
+    if (cnt == 0) return;
+    if (((m >> 15) & 3u) == 2u) {
+        walk_z<TOF>(l, G, P, r, nullptr, acc, true, b);
+        return;
+    }
+    Held h;
+    if (m & REC_INNER) walk<PASSES, 0, true, TOF, false, false>(l, G, P, r, 0, nullptr, h);
+    else walk<PASSES, 0, false, TOF, false, false>(l, G, P, r, 0, nullptr, h);
+    backward<TOF>(l, G, P, r, h, b, acc);
 }
 
 // Sums of two events over the warp in one tree: lanes 0-15 return the first

@@ -1,6 +1,7 @@
 """GPU: the standalone operators where their launch rules branch: projections
-of many events (TOF weights from a table per block) against the same events
-in small calls (an erf per sample)."""
+of many events (TOF weights from a table per block; from 16 384 events on 3D
+grids by the table projector's walk) against the same events in small calls
+(the event kernel, an erf per sample)."""
 import numpy as np
 import pytest
 
@@ -19,13 +20,26 @@ def lm():
     return _lm
 
 
-@pytest.mark.parametrize("two_d", [False, True])
-def test_many_events_equal_few(lm, two_d):
+# scanner (rings, crystals, radius, pitch), grid, voxel size, TOF bins
+PROJ = {
+    "2d": ((1, 128, 150.0, 1.0), (41, 37, 1), 5.0, 27),
+    "rows": ((8, 96, 150.0, 8.0), (41, 37, 14), 5.0, 27),
+    "bricks": ((8, 96, 150.0, 8.0), (44, 36, 14), 5.0, 27),
+    "non_tof": ((8, 96, 150.0, 8.0), (44, 36, 14), 5.0, 0),
+    "non_tof_many_planes": ((8, 96, 150.0, 8.0), (180, 36, 14), 1.0, 0),
+    "z_principal": ((60, 48, 60.0, 6.0), (24, 20, 80), 4.0, 27),
+}
+
+
+@pytest.mark.parametrize("name", sorted(PROJ))
+def test_many_events_equal_few(lm, name):
     """The table interpolates the TOF kernel to 1e-7 of its peak and erf
-    carries as much, so a projection moves by at most 4e-7 of the largest."""
-    sc = S.Scanner(1, 128, 150.0, 1.0) if two_d else S.Scanner(8, 96, 150.0, 8.0)
-    g = S.Grid((41, 37, 1 if two_d else 14), (5.0, 5.0, 5.0))
-    tof = S.tof_400ps(27, 600.0 / 27)
+    carries as much, so a projection moves by at most 4e-7 of the largest
+    per tap."""
+    (rings, xtal, radius, pitch), n_g, h, bins = PROJ[name]
+    sc = S.Scanner(rings, xtal, radius, pitch)
+    g = S.Grid(n_g, (h, h, h))
+    tof = S.tof_400ps(bins, 600.0 / 27)
     n = 90000
     ev = S.uniform_events(sc, tof, n, 5)
     geo = lm.Geometry(torch.from_numpy(sc.crystal_table()).cuda(), sc.n_rings, sc.n_xtal, g.n, g.h, g.origin, tof.sigma,
