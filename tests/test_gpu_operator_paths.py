@@ -1,12 +1,15 @@
-"""GPU: the standalone operators where their launch rules branch: projections
-of many events (TOF weights from a table per block; from 16 384 events on 3D
-grids by the table projector's walk) against the same events in small calls
-(the event kernel, an erf per sample)."""
+"""GPU: the standalone operators where their launch rules branch.  The
+sensitivity image by ring-pair profiles (rings that are copies of each other,
+z-principal ring pairs, a displaced ring, non-TOF, planes in several groups)
+against the FP64 oracle; projections of many events (TOF weights from a table
+per block; from 16 384 events on 3D grids by the table projector's walk)
+against the same events in small calls (the event kernel, an erf per sample)."""
 import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 
+import oracle as O
 from paper_2201_05497_gb300 import synth as S
 
 pytestmark = pytest.mark.gpu
@@ -18,6 +21,34 @@ def lm():
     build.build()
     _lm.load_library()
     return _lm
+
+
+# (rings, crystals, radius, pitch), grid, voxel size, TOF bins, displaced crystal
+SENS = {
+    "cylinder": ((9, 40, 100.0, 7.0), (24, 21, 16), 6.0, 15, False),
+    "non_tof": ((9, 40, 100.0, 7.0), (24, 21, 16), 6.0, 0, False),
+    "z_principal": ((20, 24, 40.0, 8.0), (16, 18, 30), 4.0, 9, False),
+    "displaced": ((6, 32, 100.0, 7.0), (20, 20, 9), 7.0, 9, True),
+    "plane_groups": ((20, 16, 150.0, 9.0), (270, 9, 20), 1.0, 9, False),
+}
+
+
+@pytest.mark.parametrize("name", sorted(SENS))
+def test_sens_matches_oracle(lm, name):
+    (rings, xtal, radius, pitch), n, h, bins, displaced = SENS[name]
+    sc = S.Scanner(rings, xtal, radius, pitch)
+    g = S.Grid(n, (h, h, h))
+    tof = (20.0, 18.0, 3.0, bins)
+    tab = sc.crystal_table().copy()
+    if displaced:
+        tab[2 * xtal + 5] += np.float32([1.5, -0.7, 0.4])
+    lf = np.random.default_rng(3).uniform(0.2, 1.0, sc.n_lor).astype(np.float32)
+    geo_o = O.Geometry(tab, rings, xtal, g.n, g.h, g.origin, tof)
+    geo_g = lm.Geometry(torch.from_numpy(tab).cuda(), rings, xtal, g.n, g.h, g.origin, *tof)
+    s_or = O.sens(geo_o, lf)
+    for ws in (True, False):
+        s = lm.sens(geo_g, torch.from_numpy(lf).cuda(), use_workspace=ws).cpu().numpy()
+        assert np.linalg.norm(s - s_or) <= 1e-5 * np.linalg.norm(s_or), ws
 
 
 # scanner (rings, crystals, radius, pitch), grid, voxel size, TOF bins
