@@ -536,6 +536,7 @@ def run_gpu(args):
             if table:
                 traffic = profiled_traffic(f"ev_table_kernel_data_update_{args.workload}.txt",
                                            ["paper_2201_05497_gb300/csrc/lm_table.cu",
+                                            "paper_2201_05497_gb300/csrc/lm_walk.cuh",
                                             "paper_2201_05497_gb300/csrc/lm_device.cuh"])
             else:
                 traffic = profiled_traffic(f"ev_kernel_data_update_{args.workload}.txt",

@@ -1150,6 +1150,58 @@ __global__ void __launch_bounds__(256, 2) image_tma_kernel(const lmh::ImgArgs A)
         if (!tma_item(A, m, u, it, A.xcur, A.x_nxt_std, A.x_nxt_yf, sm, p)) break;
 }
 
+// Image pass of a small 2D image (float accumulators of both layouts, TV):
+// one voxel per thread, so that 16 384 voxels spread over the chip (32 x 32
+// tiles of it keep 16 blocks busy, each waiting for its copies).  A prior update
+// recomputes the dual step at the two backward neighbours instead of exchanging it:
+// everything is in L2.  Same operations in the same order as the tiled passes.
+__global__ void __launch_bounds__(128) image_small_kernel(const lmh::ImgArgs A)
+{
+    const int u = A.u;
+    const PassMode m = pass_mode(A, u);
+    const int nx = A.n[0], ny = A.n[1];
+    const int64_t V = A.V;
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= V) return;
+    const int iy = (int)(j / nx), ix = (int)(j - (int64_t)iy * nx);
+    const int64_t k = (int64_t)ix * ny + iy;  // y-fastest index
+    const float x0 = A.x_cur[j], tm = A.T[j], z0 = A.z[j], zc = A.kahan ? A.zc[j] : 0.0f;
+    float dz;
+    if (m.data) {
+        // 2D traversals add to the first halves of the pairs
+        dz = A.acc_std[2 * j] + 0.0f;
+        dz += A.acc_yf[2 * k] + 0.0f;
+        A.acc_std[2 * j] = 0.0f;
+        A.acc_yf[2 * k] = 0.0f;
+    } else {
+        const float* x = A.x_cur;
+        const float f[3] = {0.0f, 0.0f, 0.0f};
+        auto dual = [&](int px, int py, float* o, float* d) {
+            const int64_t p = (int64_t)py * nx + px;
+            const float c = x[p];
+            dual_voxel(A.s_prior, A.beta, false, false, f, px < nx - 1 ? x[p + 1] - c : 0.0f,
+                       py < ny - 1 ? x[p + nx] - c : 0.0f, 0.0f, m.wc[p], m.wc[V + p], 0.0f, o, d);
+        };
+        float o[3], d[3], on[3], dl[3] = {0.0f, 0.0f, 0.0f}, du[3] = {0.0f, 0.0f, 0.0f};
+        dual(ix, iy, o, d);
+        if (ix >= 1) dual(ix - 1, iy, on, dl);
+        if (iy >= 1) dual(ix, iy - 1, on, du);
+        const_cast<float*>(m.wn)[j] = o[0];
+        const_cast<float*>(m.wn)[V + j] = o[1];
+        dz = 0.0f;
+        if (ix < nx - 1) dz -= d[0];
+        if (ix >= 1) dz += dl[0];
+        if (iy < ny - 1) dz -= d[1];
+        if (iy >= 1) dz += du[1];
+    }
+    float zh, zl;
+    const float xn = primal_step(x0, tm, z0, zc, dz, m.inv_p, A.kahan != 0, zh, zl);
+    A.z[j] = zh;
+    if (A.kahan) A.zc[j] = zl;
+    A.x_nxt_std[j] = xn;
+    if (A.x_nxt_yf != nullptr) A.x_nxt_yf[k] = xn;
+}
+
 // Batched epochs: work items (frame, column, z run) over the active frames.
 __global__ void __launch_bounds__(256, 2) image_tma_batch_kernel(const lmh::BatchImgArgs B)
 {
@@ -1755,6 +1807,17 @@ void launch_image_tma(const ImgArgs& a, cudaStream_t st)
     const int grid =
         a.xp ? 2 * num_sms() : (int)std::max<int64_t>(1, std::min<int64_t>(items, 2 * (int64_t)num_sms()));
     image_tma_kernel<<<grid, 256, TmaLayout::total, st>>>(a);
+    count_launch();
+}
+
+bool image_small(const lm_grid* g)
+{
+    return g->n[2] == 1 && g->n[0] > 1 && g->n[1] > 1 && nvox(g) <= 1 << 17;
+}
+
+void launch_image_small(const ImgArgs& a, cudaStream_t st)
+{
+    image_small_kernel<<<(a.V + 127) / 128, 128, 0, st>>>(a);
     count_launch();
 }
 

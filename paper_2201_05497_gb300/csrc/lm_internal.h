@@ -485,6 +485,10 @@ int64_t image_tiles(const lm_grid* g);
 enum { IP_INIT = 0, IP_UPDATE = 1 };
 void launch_image_pass(const ImgArgs& a, cudaStream_t st);
 void launch_image_tma(const ImgArgs& a, cudaStream_t st);
+// one voxel per thread: 2D grids of at most 2^17 voxels (float mode, TV), beyond which the tiled passes
+// have blocks enough
+bool image_small(const lm_grid* g);
+void launch_image_small(const ImgArgs& a, cudaStream_t st);
 void launch_image_tma_batch(const BatchImgArgs& b, int grid, cudaStream_t st);
 int image_tma_batch_grid(const lm_grid* g, int cap);
 int tma_zlen(const lm_grid* g);                       // z slices per TMA work item

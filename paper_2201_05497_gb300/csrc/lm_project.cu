@@ -535,7 +535,7 @@ __device__ __forceinline__ void event_chunk(const EvArgs& A, const float* __rest
     }
 }
 
-// Event kernel.  A warp takes chunks of up to `chunk` consecutive events; the
+// Event kernel.  A warp takes chunks of up to `chunk` consecutive events (see the queues below); the
 // lanes load them coalesced and each lane sets up the traversal of its own
 // event.  Groups of G lanes then process one event each (32/G events in
 // flight per warp): lane s of a group takes planes i0 + s, i0 + s + G, ...,
@@ -593,13 +593,28 @@ __global__ void __launch_bounds__(256, G == 8 ? 2 : 3) ev_kernel(const EvArgs A)
     }
     float wmax = 0.0f;
     unsigned long long cnt_s = 0, cnt_t = 0;
+    // The global counter serves one draw (and one warp's release below) in about
+    // 2.5 ns, so a launch of few chunks would wait for little else (7 143 events in
+    // chunks of 1: 18 us of draws, 9 us of releases); up to eight chunks per warp
+    // block b takes the chunks b, b + blocks, ... from a counter in shared memory.
+    __shared__ int s_next;
+    const bool global_queue = A.queue != nullptr && nchunks > 8 * total_warps;
+    const bool local_queue = A.queue != nullptr && !global_queue;
+    if (local_queue) {
+        if (threadIdx.x == 0) s_next = 0;
+        __syncthreads();
+    }
     int64_t it = 0;
     for (;;) {
         int64_t c;
-        if (A.queue != nullptr) {
+        if (global_queue) {
             unsigned long long cc = 0;
             if (lane == 0) cc = atomicAdd(A.queue, 1ULL);
             c = (int64_t)__shfl_sync(FULL, cc, 0);
+        } else if (local_queue) {
+            int k = 0;
+            if (lane == 0) k = atomicAdd(&s_next, 1);
+            c = (int64_t)__shfl_sync(FULL, k, 0) * gridDim.x + blockIdx.x;
         } else {
             c = warp_global + it * total_warps;
             ++it;
@@ -627,7 +642,7 @@ __global__ void __launch_bounds__(256, G == 8 ? 2 : 3) ev_kernel(const EvArgs A)
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
         if (lane == 0 && m > 0.0f) atomicMax(A.maxbits, __float_as_uint(m));
     }
-    if (A.queue != nullptr) {
+    if (global_queue) {
         // the last warp to finish resets the counters for the next launch
         __syncwarp();
         if (lane == 0) {

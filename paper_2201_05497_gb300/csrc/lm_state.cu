@@ -55,6 +55,7 @@ struct lm_state_s {
     unsigned* err;    // set by a bounded device wait that gave up
     bool tma;         // image passes staged by TMA (grid permitting, unless disabled)
     bool tma_data;    // TMA-staged data passes, plain prior passes (image_kernel 3)
+    bool small;       // small 2D image: one-voxel-per-thread passes (prior step fused)
     bool has_res;     // resolution model P = A G: the event kernels read G x from gx / gxyf
     float *gx, *gxyf; // G x in both layouts (float mode; scratch of the back-projection's G)
     float* rt;        // scratch image of the resolution model's passes (float mode)
@@ -167,7 +168,7 @@ void carve(lm_state* st, Carve& c, const lm_grid* g, int64_t N, int n, bool det,
 // directional TV's field read where it needs it); the plain prior pass
 // takes it from the event kernel's prior branch (which stores D = P (w+ - w)
 // for the directional TV).
-bool tma_fuses_prior(const lm_state* st) { return st->tma; }
+bool tma_fuses_prior(const lm_state* st) { return st->tma || st->small; }
 
 EvArgs base_ev_args(const lm_state* st)
 {
@@ -402,7 +403,9 @@ int launch_image_part(lm_state* st, int u, int cur, int nxt, int slot0, cudaStre
     // scale slots: update u reads slot (slot0 + u) & 1, its pass clears the other one
     im.slot0 = slot0;
     im.xcur = cur;
-    if (st->tma) {
+    if (st->small) {
+        launch_image_small(im, s);
+    } else if (st->tma) {
         launch_image_tma(im, s);
     } else if (st->tma_data) {
         // TMA-staged data passes, plain prior passes
@@ -838,6 +841,8 @@ int lmspdhg_create(lm_state** out, const lm_scanner* sc, const lm_grid* grid, co
     LM_TRY(cudaMemsetAsync(st->err, 0, 16, s));
     st->tma = false;
     st->tma_data = false;
+    st->small = P.image_kernel == 0 && image_small(grid) && !st->det && P.xi == nullptr && P.tile_buf == nullptr &&
+                !st->shard && P.epoch_kernel != 2;
     st->zlen = 1;
     st->has_res = P.res_fwhm > 0.0f;
     if (st->has_res) res_plan(grid, P.res_fwhm, st->res);  // validated above
@@ -1496,6 +1501,7 @@ void fill_slot(lm_batch* b, int s, lm_state* st)
     a.xbyf[1] = st->xyf[1];
     a.maxbits_base = st->maxbits;
     a.prior_only = st->table ? 1 : 0;  // the table kernel runs the data updates
+    a.prior_fused = st->tma ? 1 : 0;   // (a batch's passes are the tiled ones)
     if (!st->det) {
         a.acc_std = st->acc_std;
         a.acc_yf = st->acc_yf;
