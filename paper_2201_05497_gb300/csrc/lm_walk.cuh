@@ -286,6 +286,12 @@ __device__ __noinline__ float walk_z(const Lane l, const Geo& G, const lmh::Pair
     return s;
 }
 
+template <bool SAFE>
+__device__ __forceinline__ float times(float q, float b)
+{
+    return SAFE && q == 0.0f ? 0.0f : q * b;
+}
+
 // Forward part of one event.  Planes beyond the held ones (finer grids) are
 // walked sixteen at a time.
 template <bool TOF, bool SAFE = false>
@@ -311,7 +317,8 @@ __device__ __forceinline__ float forward(const Lane& l, const Geo& G, const lmh:
 }
 
 // Back-projection part of one event: b is its value times the sample length.
-template <bool TOF>
+// SAFE: nothing is added where the weight is 0 (b may be an infinity or NaN).
+template <bool TOF, bool SAFE = false>
 __device__ __forceinline__ void backward(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r,
                                          const Held& h, float b, char* acc)
 {
@@ -324,12 +331,12 @@ __device__ __forceinline__ void backward(const Lane& l, const Geo& G, const lmh:
 #pragma unroll
     for (int p = 0; p < PASSES; ++p)
         if (16 * p < cnt && h.off[p] != NONE)
-            atomicAdd(reinterpret_cast<float2*>(acc + h.off[p]), make_float2(h.q0[p] * b, h.q1[p] * b));
+            atomicAdd(reinterpret_cast<float2*>(acc + h.off[p]), make_float2(times<SAFE>(h.q0[p], b), times<SAFE>(h.q1[p], b)));
     for (int p = PASSES; 16 * p < cnt; ++p) {
         Held t;
         walk<1, 0, false, TOF, false, false>(l, G, P, r, p, nullptr, t);
         if (t.off[0] != NONE)
-            atomicAdd(reinterpret_cast<float2*>(acc + t.off[0]), make_float2(t.q0[0] * b, t.q1[0] * b));
+            atomicAdd(reinterpret_cast<float2*>(acc + t.off[0]), make_float2(times<SAFE>(t.q0[0], b), times<SAFE>(t.q1[0], b)));
     }
 }
 
@@ -347,7 +354,7 @@ __device__ __forceinline__ void spread(const Lane& l, const Geo& G, const lmh::P
     Held h;
     if (m & REC_INNER) walk<PASSES, 0, true, TOF, false, false>(l, G, P, r, 0, nullptr, h);
     else walk<PASSES, 0, false, TOF, false, false>(l, G, P, r, 0, nullptr, h);
-    backward<TOF>(l, G, P, r, h, b, acc);
+    backward<TOF, true>(l, G, P, r, h, b, acc);
 }
 
 // Sums of two events over the warp in one tree: lanes 0-15 return the first

@@ -89,3 +89,30 @@ def test_many_events_equal_few(lm, name):
     ps = torch.cat(ps)
     assert float((p - ps).abs().max()) <= 4e-7 * float(ps.abs().max()) * 4  # four taps
     assert float((b - bs).norm() / bs.norm()) <= 2e-6
+
+
+def test_non_finite_stays_with_its_weight(lm):
+    """A voxel of weight 0 does not enter a projection, nor does an event's
+    value enter a voxel of weight 0, whatever they hold: an infinite voxel
+    or value touches the same elements as with few events."""
+    sc = S.Scanner(9, 64, 150.0, 5.0)
+    g = S.Grid((44, 36, 9), (5.0, 5.0, 5.0))  # rings on slice centres: the upper neighbour's weight is often 0
+    tof = S.tof_400ps(27, 600.0 / 27)
+    n = 20000
+    ev = S.uniform_events(sc, tof, n, 8)
+    geo = lm.Geometry(torch.from_numpy(sc.crystal_table()).cuda(), sc.n_rings, sc.n_xtal, g.n, g.h, g.origin, tof.sigma,
+                      tof.bin, tof.n_sigma, tof.n_bins)
+    dev = lm.DeviceEvents.from_numpy(ev)
+    x = torch.ones(geo.V, device="cuda")
+    x[44 * 36 * 4:44 * 36 * 5] = float("inf")
+    v = torch.ones(n, device="cuda")
+    v[::1000] = float("inf")
+    p = torch.isfinite(lm.fwd(geo, x, dev))
+    b = lm.back(geo, v, dev)
+    ps, bs = [], torch.zeros(geo.V, device="cuda")
+    for s in range(0, n, 5000):
+        part = lm.DeviceEvents(*[t[s:s + 5000].contiguous() for t in (dev.det1, dev.det2, dev.tof, dev.corr, dev.contam)])
+        ps.append(torch.isfinite(lm.fwd(geo, x, part)))
+        bs = lm.back(geo, v[s:s + 5000].contiguous(), part, img=bs)
+    assert bool((p == torch.cat(ps)).all()) and not bool(p.all()) and bool(p.any())
+    assert not bool(torch.isnan(b).any()) and bool((torch.isinf(b) == torch.isinf(bs)).all())
