@@ -368,7 +368,7 @@ struct BatchTabArgs {
 };
 int launch_table_batch(const BatchTabArgs& b, cudaStream_t st);
 int trav_build(const lmk::Geo& G, const lm_events& ev, const uint16_t* mu, const float* tof_tab,
-               const TravLayout& L, char* base, cudaStream_t st);
+               const TravLayout& L, char* base, bool stored, cudaStream_t st);
 // Standalone projections by the table projector's walk: EV_FWD out[e] = c_e J_e x
 // from xp, EV_BACK acc += c_e v_e J_e^T.
 struct OpArgs {

@@ -300,7 +300,12 @@ int build_table(lm_state* st, cudaStream_t s)
     ev.corr = st->corr;
     ev.contam = st->contam;
     ev.n = st->N;
-    return trav_build(st->G, ev, st->mu, st->tof_tab, st->tv, st->tv_base, s);
+    // Which product of the TOF coordinate is rounded first (lor_setup) moves samples within an ulp of the
+    // 3-sigma cut in or out of the window, a few per 1e6 events.  Small updates of frames that leave the
+    // projector open ran the direct kernel (it was the faster one below about 64 000 events), all others the
+    // table: each keeps the samples it had.
+    const bool stored = st->P.group != 0 || st->P.trav_keep || st->sub_off_h[1] - st->sub_off_h[0] >= 65536;
+    return trav_build(st->G, ev, st->mu, st->tof_tab, st->tv, st->tv_base, stored, s);
 }
 
 // Resolution model: G x into gx (x-fastest) and gxyf (y-fastest), through the

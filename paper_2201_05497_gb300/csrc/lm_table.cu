@@ -12,11 +12,11 @@
 // Measured on the 200 x 200 x 96 grid (GB300, CUDA events around the launch),
 // one plane per lane over two image layouts and two accumulators (before) /
 // two lanes per plane over bricked z pairs: 7 143 events 17.5 / 14.1 us,
-// 357 143 events 200 / 133 us, 2.14e6 events 1.09 ms / 0.67 ms.  ncu of the
-// row layout of the pairs (before the bricks) at 357 143 events: SM-to-L2
-// request cycles 71 % of peak = one per line gathered (17.1 M) plus one per
-// sector added to (19.5 M), issue 42 %, 247 warp instructions per event (343
-// before): the requests bound it, and the bricks cut them (176 -> 134 us).
+// 357 143 events 200 / 133 us, 2.14e6 events 1.09 ms / 0.67 ms.  ncu at
+// 357 143 events: with the pairs in rows 71 % of the SM-to-L2 request cycles
+// (17.1 M lines gathered + 19.5 M sectors added to), issue 42 %, 176 us; in bricks
+// 9.2 M + 16.0 M, request cycles 65 %, issue 72 % (305 warp instructions per
+// event), 133 us: instructions and requests now bound it about equally.
 // Ordering the events by direction and place moved it by less than 10 % in
 // either direction, and one-plane-per-lane with the same pairs was no faster.
 // Per sample the positions and weights are the direct kernel's.
@@ -80,7 +80,7 @@ __device__ __forceinline__ unsigned pack_meta(int i0, int cnt, int k)
 __global__ void trav_build_kernel(const Geo G, const int32_t* __restrict__ det1, const int32_t* __restrict__ det2,
                                   const int16_t* __restrict__ tofb, const float* __restrict__ corr,
                                   const uint16_t* __restrict__ mu, int64_t N, const float* __restrict__ tab,
-                                  float4* __restrict__ r0, float4* __restrict__ r1, int2* __restrict__ meta)
+                                  float4* __restrict__ r0, float4* __restrict__ r1, int2* __restrict__ meta, bool stored)
 {
     __shared__ float s_tab[TOF_TAB_N + 1];
     for (int k = threadIdx.x; k <= TOF_TAB_N; k += blockDim.x) s_tab[k] = tab[k];
@@ -90,7 +90,7 @@ __global__ void trav_build_kernel(const Geo G, const int32_t* __restrict__ det1,
         const int d1 = det1[e], d2 = det2[e], m = (int)tofb[e];
         bool ok = d1 >= 0 && d1 < G.n_det && d2 >= 0 && d2 < G.n_det && d1 != d2 && m >= -G.M && m <= G.M;
         Lor L;
-        ok = ok && lor_setup(G, d1, d2, m, TOF_BIN, true, L, true);
+        ok = ok && lor_setup(G, d1, d2, m, TOF_BIN, true, L, stored);
         float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
         unsigned mw = 0u;
         if (ok) {
@@ -404,13 +404,14 @@ void launch_pair_image(const lm_grid* g, const PairLay& P, const float* x, float
 }
 
 int trav_build(const Geo& G, const lm_events& ev, const uint16_t* mu, const float* tof_tab, const TravLayout& L,
-               char* base, cudaStream_t st)
+               char* base, bool stored, cudaStream_t st)
 {
     LM_CHECK(G.tof_on && tof_tab != nullptr, LM_ERR_INVALID_ARG, "the traversal table needs TOF data");
     if (ev.n <= 0) return LM_OK;
     const int grid = std::max<int64_t>(1, std::min<int64_t>((ev.n + 255) / 256, (int64_t)num_sms() * 8));
     trav_build_kernel<<<grid, 256, 0, st>>>(G, ev.det1, ev.det2, ev.tof, ev.corr, mu, ev.n, tof_tab,
-                                            (float4*)(base + L.r0), (float4*)(base + L.r1), (int2*)(base + L.meta));
+                                            (float4*)(base + L.r0), (float4*)(base + L.r1), (int2*)(base + L.meta),
+                                            stored);
     count_launch();
     LM_CUDA(cudaGetLastError());
     return LM_OK;
