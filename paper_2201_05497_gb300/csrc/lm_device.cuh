@@ -304,6 +304,9 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
+// True where a float array takes 16-byte accesses at every fourth element.
+__host__ __device__ __forceinline__ bool quad_aligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 __device__ __forceinline__ float warp_sum(float v)
 {
 #pragma unroll

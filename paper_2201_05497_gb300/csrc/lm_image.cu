@@ -762,6 +762,16 @@ __device__ __forceinline__ void st_quad(float* p, const float* v)
 {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
+// Four elements of a caller's array, which may start at any float.
+__device__ __forceinline__ void ld_quad_any(const float* p, bool aligned, float* v)
+{
+    if (aligned) {
+        ld_quad(p, v);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = __ldg(p + e);
+    }
+}
 
 // The prior's dual step at one voxel (same operations as prior_voxel): w+ =
 // v / max(1, |v|/beta), v = w + S K x from the forward differences g (the
@@ -821,9 +831,10 @@ __device__ __forceinline__ void prior_slice(const lmh::ImgArgs& A, int wp, uint8
         const int xb = (ty + 1) * XHW + tx + 4, wb = (ty + 1) * WBW + tx + 4;
         float f[3][4] = {};
         if (dtv) {
-            ld_quad(xi + j, f[0]);
-            ld_quad(xi + V + j, f[1]);
-            if (hz) ld_quad(xi + 2 * V + j, f[2]);
+            const bool q = quad_aligned(xi);  // (V is a multiple of 4: so are its components)
+            ld_quad_any(xi + j, q, f[0]);
+            ld_quad_any(xi + V + j, q, f[1]);
+            if (hz) ld_quad_any(xi + 2 * V + j, q, f[2]);
         }
         float xy[4], xz[4], w[3][4] = {}, o[3][4];
         const float xr = X0[xb + 4];

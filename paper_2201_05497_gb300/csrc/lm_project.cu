@@ -230,13 +230,14 @@ __device__ __forceinline__ void prior_quad(const EvArgs& A, const float* __restr
 }
 
 // Prior dual step over voxels [j0, j1) by `nthr` threads numbered t: quads
-// when rows are a multiple of 4 long, single voxels otherwise.
+// when rows are a multiple of 4 long (and the caller's directional field, if
+// any, starts on 16 bytes), single voxels otherwise.
 __device__ __forceinline__ void prior_range(const EvArgs& A, const float* __restrict__ x, int wp, int64_t j0,
                                             int64_t j1, int64_t t, int64_t nthr)
 {
     const float* wc = A.w_cur[wp];
     float* wn = A.w_nxt[wp];
-    if ((A.G.n[0] & 3) == 0) {
+    if ((A.G.n[0] & 3) == 0 && quad_aligned(A.xi)) {
         for (int64_t j = j0 + 4 * t; j < j1; j += 4 * nthr) prior_quad(A, x, wc, wn, j);
     } else {
         for (int64_t j = j0 + t; j < j1; j += nthr) prior_voxel(A, x, wc, wn, (int)j);
