@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(256) primal_quad_kernel(const PdArgs A)
     st4(A.ubar + j, bo);
 }
 
-// One voxel per thread (rows not a multiple of 4 long).
+// One voxel per thread (rows not a multiple of 4 long, or u not on 16 bytes).
 __global__ void __launch_bounds__(256) dual_point_kernel(const PdArgs A)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -396,7 +396,8 @@ int run_pdhg(const lm_grid* g, const Ws& W, float* u, int iters, double knorm, c
     a.z = W.z;
     a.w = W.w;
     a.sc = W.sc;
-    const bool quad = (a.nx & 3) == 0;
+    // (u is the caller's array, which may start at any float; the others are the workspace's)
+    const bool quad = (a.nx & 3) == 0 && quad_aligned(u);
     const int blocks = quad ? (a.V / 4 + 255) / 256 : (a.V + 255) / 256;
     for (int k = 0; k < iters; ++k) {
         a.k = k;
