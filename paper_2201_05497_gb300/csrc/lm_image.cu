@@ -1730,13 +1730,11 @@ static EncodeTiled encoder()
     return fn;
 }
 
+// Before every launch: the attribute belongs to the current device's copy of the kernel.
 static void tma_attributes()
 {
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(image_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TmaLayout::total);
-        cudaFuncSetAttribute(image_tma_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TmaLayout::total);
-    });
+    cudaFuncSetAttribute(image_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TmaLayout::total);
+    cudaFuncSetAttribute(image_tma_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TmaLayout::total);
 }
 
 // rank <= 4; dims innermost first; strides in bytes for dims 1..rank-1

@@ -417,11 +417,19 @@ int trav_build(const Geo& G, const lm_events& ev, const uint16_t* mu, const floa
     return LM_OK;
 }
 
+// Before every launch: the attribute belongs to the current device's copy of
+// the kernel, so a flag kept by the process would serve the first device only.
+template <class F>
+static void table_smem(F* kernel)
+{
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAB_SMEM);
+}
+
 template <class F>
 static int table_blocks(F* kernel)
 {
     int b = 0;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAB_SMEM);
+    table_smem(kernel);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, TAB_THREADS, TAB_SMEM) != cudaSuccess || b < 1) b = 1;
     return num_sms() * b;
 }
@@ -440,6 +448,7 @@ int table_grid()
 
 int launch_table_batch(const BatchTabArgs& b, cudaStream_t st)
 {
+    table_smem(ev_table_batch_kernel);
     ev_table_batch_kernel<<<table_grid(), TAB_THREADS, TAB_SMEM, st>>>(b);
     count_launch();
     LM_CUDA(cudaGetLastError());
@@ -477,8 +486,14 @@ int launch_table(int mode, const TabArgs& a, cudaStream_t st)
 {
     const int grid = table_grid();
     switch (mode) {
-    case EV_DATA: ev_table_kernel<EV_DATA><<<grid, TAB_THREADS, TAB_SMEM, st>>>(a); break;
-    case EV_FWD: ev_table_kernel<EV_FWD><<<grid, TAB_THREADS, TAB_SMEM, st>>>(a); break;
+    case EV_DATA:
+        table_smem(ev_table_kernel<EV_DATA>);
+        ev_table_kernel<EV_DATA><<<grid, TAB_THREADS, TAB_SMEM, st>>>(a);
+        break;
+    case EV_FWD:
+        table_smem(ev_table_kernel<EV_FWD>);
+        ev_table_kernel<EV_FWD><<<grid, TAB_THREADS, TAB_SMEM, st>>>(a);
+        break;
     default: set_error("unknown traversal-table mode %d", mode); return LM_ERR_INVALID_ARG;
     }
     count_launch();

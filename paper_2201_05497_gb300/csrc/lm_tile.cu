@@ -752,16 +752,14 @@ int tile_build(TileArgs& A, const TileLayout& Lt, char* base, int64_t N, const s
     return LM_OK;
 }
 
+// At each state's creation: the attribute belongs to the current device's copy of the kernel.
 void tile_attributes()
 {
-    static bool done = false;
-    if (done) return;
     const size_t sm = tile_smem(TL_TZ + 1);
     cudaFuncSetAttribute(tl_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaFuncSetAttribute(tl_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaFuncSetAttribute(tl_back_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaFuncSetAttribute(tl_back_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    done = true;
 }
 
 int launch_tile_update(const TileArgs& A, bool two_d, cudaStream_t st)
