@@ -177,7 +177,6 @@ struct EvArgs {
     float beta;
     int ndim;
     const float* tof_tab;       // device table (TOF_TAB_N + 1 floats) or nullptr (erf per sample)
-    int make_tab;               // 1 without tof_tab: every block tabulates the TOF kernel itself
     int group;                  // lanes per event: 8, 16 or 32 (0 = 16)
     // batched epochs: both x buffers (index = update parity) and the scale slots
     const float* xb[2];

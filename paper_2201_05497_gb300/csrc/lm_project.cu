@@ -566,18 +566,8 @@ __global__ void __launch_bounds__(256, G == 8 ? 2 : 3) ev_kernel(const EvArgs A)
     const bool has_yf = A.x_yf != nullptr || A.acc_yf != nullptr || A.acci_yf != nullptr;
     const float* tab = nullptr;
     float inv_dt = 0.0f;
-    if (T::traverse && tofmode == TOF_BIN && (A.tof_tab != nullptr || A.make_tab)) {
-        if (A.tof_tab != nullptr) {
-            for (int k = threadIdx.x; k <= lmh::TOF_TAB_N; k += blockDim.x) s_tab[k] = A.tof_tab[k];
-        } else {
-            // the kernel is even; erfc keeps the relative accuracy of its tails
-            for (int k = threadIdx.x; k <= lmh::TOF_TAB_N / 2; k += blockDim.x) {
-                const float tau = Gm.W - (2.0f * Gm.W / (float)lmh::TOF_TAB_N) * (float)k, hb = 0.5f * Gm.bin;
-                const float w = 0.5f * (erfcf((tau - hb) * Gm.inv_s) - erfcf((tau + hb) * Gm.inv_s));
-                s_tab[k] = w;
-                s_tab[lmh::TOF_TAB_N - k] = w;
-            }
-        }
+    if (T::traverse && A.tof_tab != nullptr && tofmode == TOF_BIN) {
+        for (int k = threadIdx.x; k <= lmh::TOF_TAB_N; k += blockDim.x) s_tab[k] = A.tof_tab[k];
         __syncthreads();
         tab = s_tab;
         inv_dt = (float)lmh::TOF_TAB_N / (2.0f * Gm.W);
@@ -759,10 +749,7 @@ __global__ void __launch_bounds__(256, G == 8 ? 2 : 3) ev_batch_kernel(const lmh
     }
 }
 
-size_t ev_smem(const EvArgs& a)
-{
-    return a.tof_tab || a.make_tab ? (size_t)(lmh::TOF_TAB_N + 1) * sizeof(float) : 0;
-}
+size_t ev_smem(const EvArgs& a) { return a.tof_tab ? (size_t)(lmh::TOF_TAB_N + 1) * sizeof(float) : 0; }
 
 template <int MODE, bool TWO_D>
 int launch_mode(const EvArgs& a, int grid, cudaStream_t st)
@@ -1377,19 +1364,15 @@ static int check_events(const lm_events* ev, bool need_corr_contam)
 }
 
 // Launch shape of the standalone operators over a.e_begin .. a.e_end: the
-// widths the autotuner finds on the 2D and 3D frames; about eight chunks per
-// warp (whole 32-event chunks left a fourth round of warps three quarters idle
-// at 357 143 events and 15 of 16 warps idle at 7 143), two events at least; and
-// the TOF weights from a table that every block makes for itself (8 pairs of
-// erfc per thread) where the events are many enough to repay it: about 45
-// samples each, each otherwise two erf.
+// widths the autotuner finds on the 2D and 3D frames, and about eight chunks per
+// warp, two events at least (whole 32-event chunks left a fourth round of warps
+// three quarters idle at 357 143 events and 15 of 16 warps idle at 7 143).
 static int operator_shape(EvArgs& a, int mode, bool two_d)
 {
     a.group = two_d ? 16 : 32;
     const int grid = ev_grid_g(mode, two_d, a.group);
     const int64_t n = a.e_end - a.e_begin, c = n / ((int64_t)grid * 8 * 8);
     a.chunk = c >= 32 ? 32 : (c <= 2 ? 2 : (int)c);
-    a.make_tab = a.G.tof_on && n * 45 > (int64_t)grid * TOF_TAB_N ? 1 : 0;
     return grid;
 }
 

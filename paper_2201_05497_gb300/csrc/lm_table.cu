@@ -160,8 +160,8 @@ __device__ __forceinline__ void table_pairs(const lmh::TabArgs& A, const lmw::La
         lmw::Held h0, h1;
         float a1 = 0.0f;
         const bool two = b + 1 < nm;
-        const float a0 = lmw::forward<true>(l, A.G, A.lay, rec[b], img, h0);
-        if (two) a1 = lmw::forward<true>(l, A.G, A.lay, rec[b + 1], img, h1);
+        const float a0 = lmw::forward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b], img, h0);
+        if (two) a1 = lmw::forward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b + 1], img, h1);
         const lmw::Rec& R = rec[b + (two ? lane >> 4 : 0)];
         const float4 dd = R.d;
         const bool valid = lane < 16 || two;
@@ -180,8 +180,8 @@ __device__ __forceinline__ void table_pairs(const lmh::TabArgs& A, const lmw::La
         float bval = R.g1.z * (yp - dd.z);                    // c step (y+ - y) / mu
         if (!valid) bval = 0.0f;
         const float b0 = __shfl_sync(FULL, bval, 0), b1 = __shfl_sync(FULL, bval, 16);
-        if (b0 != 0.0f) lmw::backward<true>(l, A.G, A.lay, rec[b], h0, b0, acc);
-        if (b1 != 0.0f) lmw::backward<true>(l, A.G, A.lay, rec[b + 1], h1, b1, acc);
+        if (b0 != 0.0f) lmw::backward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b], h0, b0, acc);
+        if (b1 != 0.0f) lmw::backward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b + 1], h1, b1, acc);
     }
     __syncwarp();
 }
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_kernel(const __grid_c
     if (threadIdx.x == 0) s_next = TAB_WARPS;
     lmw::fill_tab(s_tab, A.tof_tab);
     __syncthreads();
-    const lmw::Lane l = lmw::make_lane(s_tab, A.G.W);
+    const lmw::Lane l = lmw::table_lane(s_tab, A.G.W);
     while (c < nch) {
         table_pairs<MODE>(A, l, eb + c * CH, nm, rec);
         int k = 0;
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_batch_kernel(const __
     }
     __syncthreads();
     const long long total = s_pre[cap];
-    const lmw::Lane l = lmw::make_lane(s_tab, B.tof_W);
+    const lmw::Lane l = lmw::table_lane(s_tab, B.tof_W);
     lmw::Rec* rec = reinterpret_cast<lmw::Rec*>(s_tab + lmw::TAB_PAD) + (threadIdx.x >> 5) * 32;
     for (;;) {
         int k = 0;
@@ -285,22 +285,26 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_batch_kernel(const __
 // Standalone projections (lm_fwd, lm_back) by the same walk, the traversals set
 // up by the staging lanes.  357 143 events on the 200 x 200 x 96 grid, whole calls
 // (with the pair image, or the accumulator's clearing and fold): ev_kernel / this:
-// forward 165 / 127 us, back 317 / 141 us.
-template <int MODE, bool TOF>
+// forward 165 / 124 us, back 317 / 144 us.
+constexpr size_t OP_RECS = (size_t)TAB_WARPS * 32 * sizeof(lmw::Rec);
+constexpr size_t OP_SMEM = OP_RECS + (lmw::SERIES_N + 1) * sizeof(float4);  // TOF_SERIES; the others: OP_RECS
+
+template <int MODE, lmw::Tof TOF>
 __global__ void __launch_bounds__(TAB_THREADS, 2) op_walk_kernel(const __grid_constant__ lmh::OpArgs A)
 {
+    constexpr bool TOF_ON = TOF != lmw::NO_TOF;
     extern __shared__ float4 s_dyn[];
     __shared__ int s_next;
-    float2* s_tab = reinterpret_cast<float2*>(s_dyn);
+    float4* s_ser = s_dyn + OP_RECS / sizeof(float4);
     const Geo& G = A.G;
     const int lane = threadIdx.x & 31;
     const int CH = lmw::chunk_of(A.n, (int64_t)gridDim.x * TAB_WARPS);
     const int64_t nch = (A.n + CH - 1) / CH;
-    lmw::Rec* rec = reinterpret_cast<lmw::Rec*>(s_tab + lmw::TAB_PAD) + (threadIdx.x >> 5) * 32;
+    lmw::Rec* rec = reinterpret_cast<lmw::Rec*>(s_dyn) + (threadIdx.x >> 5) * 32;
     if (threadIdx.x == 0) s_next = 0;
-    if (TOF) lmw::make_tab(s_tab, G);
+    if (TOF == lmw::TOF_SERIES) lmw::make_series(s_ser, G);
     else __syncthreads();
-    const lmw::Lane l = lmw::make_lane(s_tab, G.W);
+    const lmw::Lane l = lmw::op_lane(s_ser, G);
     const char* img = reinterpret_cast<const char*>(A.xp);
     char* acc = reinterpret_cast<char*>(A.acc);
     for (;;) {
@@ -312,11 +316,11 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) op_walk_kernel(const __grid_co
         const int nev = (int)min((int64_t)CH, A.n - e0);
         if (lane < nev) {
             const int64_t e = e0 + lane;
-            const int d1 = A.det1[e], d2 = A.det2[e], m = TOF ? (int)A.tof[e] : 0;
-            bool ok = d1 >= 0 && d1 < G.n_det && d2 >= 0 && d2 < G.n_det && d1 != d2 && (!TOF || (m >= -G.M && m <= G.M));
+            const int d1 = A.det1[e], d2 = A.det2[e], m = TOF_ON ? (int)A.tof[e] : 0;
+            bool ok = d1 >= 0 && d1 < G.n_det && d2 >= 0 && d2 < G.n_det && d1 != d2 && (!TOF_ON || (m >= -G.M && m <= G.M));
             Lor L;
             bool inner = false;
-            ok = ok && lor_setup(G, d1, d2, m, TOF ? TOF_BIN : TOF_NONE, false, L);
+            ok = ok && lor_setup(G, d1, d2, m, TOF_ON ? TOF_BIN : TOF_NONE, false, L);
             if (ok) lmw::trim(G, L, &inner);
             lmw::Rec& r = rec[lane];
             if (ok) lmw::rec_path(make_float4(L.ua0, L.sa, L.ub0, L.sb), L.tau0, L.dtau, L.i0, L.cnt, L.k, inner, lane, r);
@@ -456,22 +460,30 @@ int launch_table_batch(const BatchTabArgs& b, cudaStream_t st)
 }
 
 template <class F>
-static int launch_op_kernel(F* kernel, const OpArgs& a, cudaStream_t st)
+static int launch_op_kernel(F* kernel, size_t smem, const OpArgs& a, cudaStream_t st)
 {
-    const int grid = table_blocks(kernel);
-    kernel<<<grid, TAB_THREADS, TAB_SMEM, st>>>(a);
+    int b = 0;
+    LM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, TAB_THREADS, smem) != cudaSuccess || b < 1) b = 1;
+    kernel<<<num_sms() * b, TAB_THREADS, smem, st>>>(a);
     count_launch();
     LM_CUDA(cudaGetLastError());
     return LM_OK;
 }
 
+template <int MODE>
+static int launch_op_mode(const OpArgs& a, cudaStream_t st)
+{
+    if (!a.G.tof_on) return launch_op_kernel(op_walk_kernel<MODE, lmw::NO_TOF>, OP_RECS, a, st);
+    const float sigmas = a.G.W * a.G.inv_s * 1.41421356f;
+    return sigmas <= lmw::SERIES_SIGMAS * 1.00001f
+               ? launch_op_kernel(op_walk_kernel<MODE, lmw::TOF_SERIES>, OP_SMEM, a, st)
+               : launch_op_kernel(op_walk_kernel<MODE, lmw::TOF_ERF>, OP_RECS, a, st);
+}
+
 int launch_op(int mode, const OpArgs& a, cudaStream_t st)
 {
-    if (mode == EV_FWD)
-        return a.G.tof_on ? launch_op_kernel(op_walk_kernel<EV_FWD, true>, a, st)
-                          : launch_op_kernel(op_walk_kernel<EV_FWD, false>, a, st);
-    return a.G.tof_on ? launch_op_kernel(op_walk_kernel<EV_BACK, true>, a, st)
-                      : launch_op_kernel(op_walk_kernel<EV_BACK, false>, a, st);
+    return mode == EV_FWD ? launch_op_mode<EV_FWD>(a, st) : launch_op_mode<EV_BACK>(a, st);
 }
 
 void launch_pair_fold(const lm_grid* g, const PairLay& P, float* img, const float* acc, cudaStream_t st)
