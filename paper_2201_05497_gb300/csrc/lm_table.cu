@@ -115,12 +115,18 @@ __global__ void trav_build_kernel(const Geo G, const int32_t* __restrict__ det1,
     }
 }
 
+// Staged events of a chunk: the first `main` are x- or y-principal, the others
+// up to `all` z-principal.
+struct Staged {
+    int main, all;
+};
+
 // Stages the events [e0, e0 + nev) that have samples into `rec` (lanes load
 // their event's entry and fields coalesced, with the streaming cache policy:
-// each is read once per update) and returns their number.  MODE EV_FWD also
-// stages the events without samples (their projection is 0).
+// each is read once per update).  MODE EV_FWD also stages the events without
+// samples (their projection is 0).
 template <int MODE>
-__device__ __forceinline__ int stage(const lmh::TabArgs& A, int64_t e0, int nev, lmw::Rec* rec)
+__device__ __forceinline__ Staged stage(const lmh::TabArgs& A, int64_t e0, int nev, lmw::Rec* rec)
 {
     const int lane = threadIdx.x & 31;
     const int64_t e = e0 + lane;
@@ -128,10 +134,11 @@ __device__ __forceinline__ int stage(const lmh::TabArgs& A, int64_t e0, int nev,
     const int2 mt = in ? __ldcs(A.meta + e) : make_int2(0, 0);
     const unsigned mw = (unsigned)mt.x;
     const unsigned cnt = (mw >> 15) & 0x7FFFu;
-    const bool mine = in && (MODE != lmh::EV_DATA || cnt != 0u);
-    const unsigned mask = __ballot_sync(FULL, mine);
+    const bool mine = in && (MODE != lmh::EV_DATA || cnt != 0u), zp = (mw >> 30) == 2u;
+    const unsigned mask = __ballot_sync(FULL, mine && !zp), zmask = __ballot_sync(FULL, mine && zp);
     if (mine) {
-        lmw::Rec& r = rec[__popc(mask & ((1u << lane) - 1u))];
+        const unsigned below = (1u << lane) - 1u;
+        lmw::Rec& r = rec[zp ? __popc(mask) + __popc(zmask & below) : __popc(mask & below)];
         const float4 g1 = __ldcs(A.r1 + e);
         const float mu = __int_as_float(mt.y), step = fabsf(g1.z);
         const float cs = (A.corr ? __ldcs(A.corr + e) : 1.0f) * step;
@@ -143,25 +150,33 @@ __device__ __forceinline__ int stage(const lmh::TabArgs& A, int64_t e0, int nev,
                           MODE == lmh::EV_DATA ? __ldcs(A.y + e) : 0.0f, mu);
     }
     __syncwarp();
-    return __popc(mask);
+    return {__popc(mask), __popc(mask) + __popc(zmask)};
 }
 
-// The staged events of one chunk, two at a time: forward projection of both,
-// one reduction, the per-event step (MODE EV_DATA: Eq. (proxD); EV_FWD: the
-// projection itself) in a half-warp each, and the back-projection of both.
-template <int MODE>
-__device__ __forceinline__ void table_pairs(const lmh::TabArgs& A, const lmw::Lane& l, int64_t e0, int nm,
+// Staged events [lo, hi), two at a time: forward projection of both, one
+// reduction, the per-event step (MODE EV_DATA: Eq. (proxD); EV_FWD: the
+// projection itself) in a half-warp each, and the back-projection of both.  Z:
+// z-principal events.  They have a loop of their own because a call or a
+// second walk in this one costs all events registers (64 per thread, and an
+// event's samples take 12): spilling them made an update 12 to 50 % longer.
+template <int MODE, bool Z>
+__device__ __forceinline__ void table_pairs(const lmh::TabArgs& A, const lmw::Lane& l, int64_t e0, int lo, int hi,
                                             const lmw::Rec* rec)
 {
     const int lane = threadIdx.x & 31;
     const char* img = reinterpret_cast<const char*>(A.xp);
     char* acc = reinterpret_cast<char*>(A.acc);
-    for (int b = 0; b < nm; b += 2) {
+    for (int b = lo; b < hi; b += 2) {
         lmw::Held h0, h1;
-        float a1 = 0.0f;
-        const bool two = b + 1 < nm;
-        const float a0 = lmw::forward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b], img, h0);
-        if (two) a1 = lmw::forward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b + 1], img, h1);
+        float a0, a1 = 0.0f;
+        const bool two = b + 1 < hi;
+        if (Z) {
+            a0 = lmw::walk_z<lmw::TOF_TABLE, false, 2>(l, A.G, A.lay, rec[b], img, nullptr, 0.0f);
+            if (two) a1 = lmw::walk_z<lmw::TOF_TABLE, false, 2>(l, A.G, A.lay, rec[b + 1], img, nullptr, 0.0f);
+        } else {
+            a0 = lmw::forward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b], img, h0);
+            if (two) a1 = lmw::forward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b + 1], img, h1);
+        }
         const lmw::Rec& R = rec[b + (two ? lane >> 4 : 0)];
         const float4 dd = R.d;
         const bool valid = lane < 16 || two;
@@ -180,9 +195,22 @@ __device__ __forceinline__ void table_pairs(const lmh::TabArgs& A, const lmw::La
         float bval = R.g1.z * (yp - dd.z);                    // c step (y+ - y) / mu
         if (!valid) bval = 0.0f;
         const float b0 = __shfl_sync(FULL, bval, 0), b1 = __shfl_sync(FULL, bval, 16);
-        if (b0 != 0.0f) lmw::backward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b], h0, b0, acc);
-        if (b1 != 0.0f) lmw::backward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b + 1], h1, b1, acc);
+        if (Z) {
+            if (b0 != 0.0f) lmw::walk_z<lmw::TOF_TABLE, true, 2>(l, A.G, A.lay, rec[b], nullptr, acc, b0);
+            if (b1 != 0.0f) lmw::walk_z<lmw::TOF_TABLE, true, 2>(l, A.G, A.lay, rec[b + 1], nullptr, acc, b1);
+        } else {
+            if (b0 != 0.0f) lmw::backward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b], h0, b0, acc);
+            if (b1 != 0.0f) lmw::backward<lmw::TOF_TABLE>(l, A.G, A.lay, rec[b + 1], h1, b1, acc);
+        }
     }
+}
+
+template <int MODE>
+__device__ __forceinline__ void table_chunk(const lmh::TabArgs& A, const lmw::Lane& l, int64_t e0, const Staged& n,
+                                            const lmw::Rec* rec)
+{
+    table_pairs<MODE, false>(A, l, e0, 0, n.main, rec);
+    table_pairs<MODE, true>(A, l, e0, n.main, n.all, rec);
     __syncwarp();
 }
 
@@ -213,17 +241,18 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_kernel(const __grid_c
     const int warp = threadIdx.x >> 5;
     lmw::Rec* rec = reinterpret_cast<lmw::Rec*>(s_tab + lmw::TAB_PAD) + warp * 32;
     int64_t c = (int64_t)warp * gridDim.x + blockIdx.x;
-    int nm = c < nch ? stage<MODE>(A, eb + c * CH, (int)min((int64_t)CH, count - c * CH), rec) : 0;
+    Staged n = {0, 0};
+    if (c < nch) n = stage<MODE>(A, eb + c * CH, (int)min((int64_t)CH, count - c * CH), rec);
     if (threadIdx.x == 0) s_next = TAB_WARPS;
     lmw::fill_tab(s_tab, A.tof_tab);
     __syncthreads();
     const lmw::Lane l = lmw::table_lane(s_tab, A.G.W);
     while (c < nch) {
-        table_pairs<MODE>(A, l, eb + c * CH, nm, rec);
+        table_chunk<MODE>(A, l, eb + c * CH, n, rec);
         int k = 0;
         if ((threadIdx.x & 31) == 0) k = atomicAdd(&s_next, 1);
         c = (int64_t)__shfl_sync(FULL, k, 0) * gridDim.x + blockIdx.x;
-        if (c < nch) nm = stage<MODE>(A, eb + c * CH, (int)min((int64_t)CH, count - c * CH), rec);
+        if (c < nch) n = stage<MODE>(A, eb + c * CH, (int)min((int64_t)CH, count - c * CH), rec);
     }
 }
 
@@ -277,8 +306,8 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_batch_kernel(const __
         while (s_pre[s + 1] <= c) ++s;
         const lmh::TabArgs& A = B.slots[s];
         const int64_t e0 = s_eb[s] + (c - s_pre[s]) * CH;
-        const int nm = stage<lmh::EV_DATA>(A, e0, (int)min((long long)CH, s_ee[s] - e0), rec);
-        table_pairs<lmh::EV_DATA>(A, l, e0, nm, rec);
+        const Staged n = stage<lmh::EV_DATA>(A, e0, (int)min((long long)CH, s_ee[s] - e0), rec);
+        table_chunk<lmh::EV_DATA>(A, l, e0, n, rec);
     }
 }
 
@@ -331,11 +360,10 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) op_walk_kernel(const __grid_co
         __syncwarp();
         for (int b = 0; b < nev; b += 2) {
             const bool two = b + 1 < nev;
-            lmw::Held h0, h1;
             if (MODE == lmh::EV_FWD) {
                 float a1 = 0.0f;
-                const float a0 = lmw::forward<TOF, true>(l, G, A.lay, rec[b], img, h0);
-                if (two) a1 = lmw::forward<TOF, true>(l, G, A.lay, rec[b + 1], img, h1);
+                const float a0 = lmw::gather<TOF>(l, G, A.lay, rec[b], img);
+                if (two) a1 = lmw::gather<TOF>(l, G, A.lay, rec[b + 1], img);
                 const float J = lmw::reduce2(a0, a1);
                 const int w = lane >> 4;
                 if ((lane & 15) == 0 && (w == 0 || two)) A.out[e0 + b + w] = rec[b + w].d.x * J;

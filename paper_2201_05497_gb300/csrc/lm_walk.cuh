@@ -316,38 +316,67 @@ __device__ __forceinline__ float walk(const Lane& l, const Geo& G, const lmh::Pa
 }
 
 // A z-principal event (B along y: its neighbours are two rows, each the first
-// half of a pair).  Adds to acc if `back`, else returns the lane's part of
-// sum w x / (c_e step).  Rare: a scanner's lines are mostly transaxial.
-template <Tof TOF>
-__device__ __noinline__ float walk_z(const Lane l, const Geo& G, const lmh::PairLay& P, const Rec& r,
-                                     const char* __restrict__ img, char* acc, bool back, float b)
+// half of a pair).  BACK: adds b times the weights to acc, else returns the
+// lane's part of sum w x / (c_e step).  Few events of a short scanner, most of
+// one that is longer than wide: U planes per lane at a time, so that 2 U gathers
+// are in flight.
+template <Tof TOF, bool BACK, int U>
+__device__ __forceinline__ float walk_z(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r,
+                                        const char* __restrict__ img, char* acc, float b)
 {
-    const int cnt = (int)(r.meta & 0x7FFFu);
+    const float4 g0 = r.g0;
+    const float tau0 = r.g1.x, dtau = r.g1.y;
+    const int cnt = (int)(r.meta & 0x7FFFu), i0 = r.i0;
     const AxisLay ax = {P.x1, P.x2, P.x3}, ay = {P.y1, P.y2, P.y3};
     float s = 0.0f;
-    for (int j = l.pl; j < cnt; j += 16) {
-        const float fi = (float)(r.i0 + j);
-        const float w = TOF == TOF_TABLE    ? tof_at(l, r.g1.x, r.g1.y, fi)
-                        : TOF == TOF_SERIES ? tof_series(l, r.g1.x, r.g1.y, fi)
-                        : TOF == TOF_ERF    ? tof_weight(G, TOF_BIN, fmaf(fi, r.g1.y, r.g1.x))
-                                            : 1.0f;
-        const float ua = fmaf(fi, r.g0.y, r.g0.x), fla = floorf(ua);
-        const float ub = fmaf(fi, r.g0.w, r.g0.z), flb = floorf(ub);
-        const int ia = (int)fla + l.par, ib = (int)flb;
-        if ((unsigned)ia >= (unsigned)G.n[0]) continue;
-        const float wa = fmaf(l.sgn, ua - fla, l.off) * w;
-        const unsigned o = along(ax, (unsigned)ia) + (unsigned)(r.i0 + j) * P.zs;
+    for (int j0 = 0; j0 < cnt; j0 += 16 * U) {
+        unsigned o0[U], o1[U];
+        float q0[U], q1[U];
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int iy = ib + e;
-            const float q = wa * (e ? ub - flb : 1.0f - (ub - flb));
-            if ((unsigned)iy >= (unsigned)G.n[1] || q == 0.0f) continue;
-            const unsigned off = o + along(ay, (unsigned)iy);
-            if (back) atomicAdd(reinterpret_cast<float*>(acc + off), q * b);
-            else s = fmaf(q, __ldg(reinterpret_cast<const float*>(img + off)), s);
+        for (int p = 0; p < U; ++p) {
+            const int jp = j0 + 16 * p + l.pl, j = min(jp, cnt - 1);  // (keeps the table index in range)
+            const float fi = (float)(i0 + j);
+            const float w = TOF == TOF_TABLE    ? tof_at(l, tau0, dtau, fi)
+                            : TOF == TOF_SERIES ? tof_series(l, tau0, dtau, fi)
+                            : TOF == TOF_ERF    ? tof_weight(G, TOF_BIN, fmaf(fi, dtau, tau0))
+                                                : 1.0f;
+            const float ua = fmaf(fi, g0.y, g0.x), fla = floorf(ua);
+            const float ub = fmaf(fi, g0.w, g0.z), flb = floorf(ub), fb = ub - flb;
+            const int ia = (int)fla + l.par, iy = (int)flb;
+            const bool in = jp < cnt && (unsigned)ia < (unsigned)G.n[0];
+            const float wa = fmaf(l.sgn, ua - fla, l.off) * w;
+            q0[p] = in && (unsigned)iy < (unsigned)G.n[1] ? wa * (1.0f - fb) : 0.0f;
+            q1[p] = in && (unsigned)(iy + 1) < (unsigned)G.n[1] ? wa * fb : 0.0f;
+            const unsigned o = along(ax, (unsigned)ia) + (unsigned)(i0 + j) * P.zs;
+            o0[p] = o + along(ay, (unsigned)iy);
+            o1[p] = o + along(ay, (unsigned)iy + 1u);
+        }
+        if (BACK) {
+#pragma unroll
+            for (int p = 0; p < U; ++p) {
+                if (q0[p] != 0.0f) atomicAdd(reinterpret_cast<float*>(acc + o0[p]), q0[p] * b);
+                if (q1[p] != 0.0f) atomicAdd(reinterpret_cast<float*>(acc + o1[p]), q1[p] * b);
+            }
+        } else {
+            float x0[U], x1[U];
+#pragma unroll
+            for (int p = 0; p < U; ++p) {
+                x0[p] = q0[p] != 0.0f ? __ldg(reinterpret_cast<const float*>(img + o0[p])) : 0.0f;
+                x1[p] = q1[p] != 0.0f ? __ldg(reinterpret_cast<const float*>(img + o1[p])) : 0.0f;
+            }
+#pragma unroll
+            for (int p = 0; p < U; ++p) s = fmaf(q1[p], x1[p], fmaf(q0[p], x0[p], s));
         }
     }
     return s;
+}
+
+// The same as a call, for kernels that meet such events among the others.
+template <Tof TOF, bool BACK>
+__device__ __noinline__ float walk_z_call(const Lane l, const Geo& G, const lmh::PairLay& P, const Rec& r,
+                                          const char* __restrict__ img, char* acc, float b)
+{
+    return walk_z<TOF, BACK, 4>(l, G, P, r, img, acc, b);
 }
 
 template <bool SAFE>
@@ -356,8 +385,10 @@ __device__ __forceinline__ float times(float q, float b)
     return SAFE && q == 0.0f ? 0.0f : q * b;
 }
 
-// Forward part of one event.  Planes beyond the held ones (finer grids) are
-// walked sixteen at a time.
+__device__ __forceinline__ bool z_principal(const Rec& r) { return ((r.meta >> 15) & 3u) == 2u; }
+
+// Forward part of one x- or y-principal event.  Planes beyond the held ones
+// (finer grids) are walked sixteen at a time.
 template <Tof TOF, bool SAFE = false>
 __device__ __forceinline__ float forward(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r,
                                          const char* __restrict__ img, Held& h)
@@ -365,7 +396,6 @@ __device__ __forceinline__ float forward(const Lane& l, const Geo& G, const lmh:
     const unsigned m = r.meta;
     const int cnt = (int)(m & 0x7FFFu);
     if (cnt == 0) return 0.0f;
-    if (((m >> 15) & 3u) == 2u) return walk_z<TOF>(l, G, P, r, img, nullptr, false, 0.0f);
     float acc;
     if ((m & REC_INNER) && cnt > 32) {
         if (cnt > 48) acc = walk<4, 3, true, TOF, true, SAFE>(l, G, P, r, 0, img, h);
@@ -380,18 +410,13 @@ __device__ __forceinline__ float forward(const Lane& l, const Geo& G, const lmh:
     return acc;
 }
 
-// Back-projection part of one event: b is its value times the sample length.
+// Back-projection part of one x- or y-principal event: b is its value times the sample length.
 // SAFE: nothing is added where the weight is 0 (b may be an infinity or NaN).
 template <Tof TOF, bool SAFE = false>
 __device__ __forceinline__ void backward(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r,
                                          const Held& h, float b, char* acc)
 {
-    const unsigned m = r.meta;
-    const int cnt = (int)(m & 0x7FFFu);
-    if (((m >> 15) & 3u) == 2u) {
-        walk_z<TOF>(l, G, P, r, nullptr, acc, true, b);
-        return;
-    }
+    const int cnt = (int)(r.meta & 0x7FFFu);
 #pragma unroll
     for (int p = 0; p < PASSES; ++p)
         if (16 * p < cnt && h.off[p] != NONE)
@@ -404,15 +429,25 @@ __device__ __forceinline__ void backward(const Lane& l, const Geo& G, const lmh:
     }
 }
 
-// Back-projection of one event that was not walked forward before.
+// Projection of one event of any principal axis.
+template <Tof TOF>
+__device__ __forceinline__ float gather(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r,
+                                        const char* __restrict__ img)
+{
+    Held h;
+    return z_principal(r) ? walk_z_call<TOF, false>(l, G, P, r, img, nullptr, 0.0f)
+                          : forward<TOF, true>(l, G, P, r, img, h);
+}
+
+// Back-projection of one event of any principal axis that was not walked forward before.
 template <Tof TOF>
 __device__ __forceinline__ void spread(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r, float b, char* acc)
 {
     const unsigned m = r.meta;
     const int cnt = (int)(m & 0x7FFFu);
     if (cnt == 0) return;
-    if (((m >> 15) & 3u) == 2u) {
-        walk_z<TOF>(l, G, P, r, nullptr, acc, true, b);
+    if (z_principal(r)) {
+        walk_z_call<TOF, true>(l, G, P, r, nullptr, acc, b);
         return;
     }
     Held h;
