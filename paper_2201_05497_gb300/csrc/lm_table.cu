@@ -159,9 +159,12 @@ __device__ __forceinline__ Staged stage(const lmh::TabArgs& A, int64_t e0, int n
 // z-principal events.  They have a loop of their own because a call or a
 // second walk in this one costs all events registers (64 per thread, and an
 // event's samples take 12): spilling them made an update 12 to 50 % longer.
+// An event with a value that is not finite is left undone and *bad set: a voxel of
+// weight 0 may hold an infinity (see table_again; walk_z reads and writes no
+// such voxels).  A projection that is not finite leaves no finite dual change.
 template <int MODE, bool Z>
 __device__ __forceinline__ void table_pairs(const lmh::TabArgs& A, const lmw::Lane& l, int64_t e0, int lo, int hi,
-                                            const lmw::Rec* rec)
+                                            const lmw::Rec* rec, int* bad)
 {
     const int lane = threadIdx.x & 31;
     const char* img = reinterpret_cast<const char*>(A.xp);
@@ -185,15 +188,18 @@ __device__ __forceinline__ void table_pairs(const lmh::TabArgs& A, const lmw::La
         const int64_t e = e0 + (R.meta >> 20);
         if (MODE == lmh::EV_FWD) {
             if (first) A.out[e] = dd.x * J;
+            if (!Z && !lmw::finite(J)) *bad = 1;
             continue;
         }
         // dual step of Eq. (proxD) with the listmode step mu_e S_e
         const float Se = R.g1.w;
         const float a = fmaf(Se, fmaf(dd.x, J, dd.y), dd.z);  // y + S (P^LM x + s)
         const float yp = prox_dstar(a, dd.w * Se);
-        if (first) __stcs(A.y + e, yp);
+        const bool ok = Z || lmw::finite(yp);
+        if (first && ok) __stcs(A.y + e, yp);
         float bval = R.g1.z * (yp - dd.z);                    // c step (y+ - y) / mu
-        if (!valid) bval = 0.0f;
+        if (!valid || !ok) bval = 0.0f;
+        if (!ok) *bad = 1;
         const float b0 = __shfl_sync(FULL, bval, 0), b1 = __shfl_sync(FULL, bval, 16);
         if (Z) {
             if (b0 != 0.0f) lmw::walk_z<lmw::TOF_TABLE, true, 2>(l, A.G, A.lay, rec[b], nullptr, acc, b0);
@@ -205,12 +211,43 @@ __device__ __forceinline__ void table_pairs(const lmh::TabArgs& A, const lmw::La
     }
 }
 
+// Once more through a chunk for the events that table_pairs left undone, those
+// whose dual step is still not finite, one at a time, without the voxels of weight
+// 0 in either direction.  Run by a block that met such an event, after its last
+// chunk, and as little code as does it: inside the loop over the chunks its
+// registers, or a call's, cost every event 12 to 25 %.
 template <int MODE>
-__device__ __forceinline__ void table_chunk(const lmh::TabArgs& A, const lmw::Lane& l, int64_t e0, const Staged& n,
+__device__ __forceinline__ void table_again(const lmh::TabArgs& A, const lmw::Lane& l, int64_t e0, int n,
                                             const lmw::Rec* rec)
 {
-    table_pairs<MODE, false>(A, l, e0, 0, n.main, rec);
-    table_pairs<MODE, true>(A, l, e0, n.main, n.all, rec);
+#pragma unroll 1
+    for (int b = 0; b < n; ++b) {
+        const lmw::Rec& R = rec[b];
+        const int64_t e = e0 + (R.meta >> 20);
+        const bool first = (threadIdx.x & 31) == 0;
+        float plain, safe, v;
+        lmw::forward_both<lmw::TOF_TABLE>(l, A.G, A.lay, R, reinterpret_cast<const char*>(A.xp), plain, safe);
+        plain = warp_sum(plain);
+        safe = warp_sum(safe);
+        if (MODE == lmh::EV_FWD) {
+            if (first && !lmw::finite(plain)) A.out[e] = R.d.x * safe;
+            continue;
+        }
+        if (lmw::finite(prox_dstar(fmaf(R.g1.w, fmaf(R.d.x, plain, R.d.y), R.d.z), R.d.w * R.g1.w))) continue;
+        const float yp = prox_dstar(fmaf(R.g1.w, fmaf(R.d.x, safe, R.d.y), R.d.z), R.d.w * R.g1.w);
+        if (first) __stcs(A.y + e, yp);
+        v = R.g1.z * (yp - R.d.z);
+        if (v != 0.0f) lmw::spread_small<lmw::TOF_TABLE>(l, A.G, A.lay, R, v, reinterpret_cast<char*>(A.acc));
+    }
+    __syncwarp();
+}
+
+template <int MODE>
+__device__ __forceinline__ void table_chunk(const lmh::TabArgs& A, const lmw::Lane& l, int64_t e0, const Staged& n,
+                                            const lmw::Rec* rec, int* bad)
+{
+    table_pairs<MODE, false>(A, l, e0, 0, n.main, rec, bad);
+    table_pairs<MODE, true>(A, l, e0, n.main, n.all, rec, bad);
     __syncwarp();
 }
 
@@ -226,7 +263,7 @@ template <int MODE>
 __global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_kernel(const __grid_constant__ lmh::TabArgs A)
 {
     extern __shared__ float4 s_dyn[];
-    __shared__ int s_next;
+    __shared__ int s_next, s_bad;
     float2* s_tab = reinterpret_cast<float2*>(s_dyn);
     int64_t eb = A.e_begin, ee = A.e_end;
     if (A.seq != nullptr) {
@@ -243,17 +280,26 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_kernel(const __grid_c
     int64_t c = (int64_t)warp * gridDim.x + blockIdx.x;
     Staged n = {0, 0};
     if (c < nch) n = stage<MODE>(A, eb + c * CH, (int)min((int64_t)CH, count - c * CH), rec);
-    if (threadIdx.x == 0) s_next = TAB_WARPS;
+    if (threadIdx.x == 0) {
+        s_next = TAB_WARPS;
+        s_bad = 0;
+    }
     lmw::fill_tab(s_tab, A.tof_tab);
     __syncthreads();
     const lmw::Lane l = lmw::table_lane(s_tab, A.G.W);
     while (c < nch) {
-        table_chunk<MODE>(A, l, eb + c * CH, n, rec);
+        table_chunk<MODE>(A, l, eb + c * CH, n, rec, &s_bad);
         int k = 0;
         if ((threadIdx.x & 31) == 0) k = atomicAdd(&s_next, 1);
         c = (int64_t)__shfl_sync(FULL, k, 0) * gridDim.x + blockIdx.x;
         if (c < nch) n = stage<MODE>(A, eb + c * CH, (int)min((int64_t)CH, count - c * CH), rec);
     }
+    __syncthreads();
+    if (s_bad)
+        for (c = (int64_t)warp * gridDim.x + blockIdx.x; c < nch; c += (int64_t)TAB_WARPS * gridDim.x) {
+            n = stage<MODE>(A, eb + c * CH, (int)min((int64_t)CH, count - c * CH), rec);
+            table_again<MODE>(A, l, eb + c * CH, n.main, rec);
+        }
 }
 
 // The data updates of every active frame of a batch at update u, from their
@@ -267,7 +313,7 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_batch_kernel(const __
     __shared__ long long s_pre[lmh::BATCH_MAX + 1];
     __shared__ long long s_eb[lmh::BATCH_MAX];
     __shared__ long long s_ee[lmh::BATCH_MAX];
-    __shared__ int s_next;
+    __shared__ int s_next, s_bad;
     const int cap = B.cap;
     if (threadIdx.x < cap) {
         const int s = threadIdx.x;
@@ -283,7 +329,7 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_batch_kernel(const __
         s_eb[s] = eb;
         s_ee[s] = ee;
     }
-    if (threadIdx.x == 0) s_next = 0;
+    if (threadIdx.x == 0) s_next = s_bad = 0;
     lmw::fill_tab(s_tab, B.tof_tab);
     __syncthreads();
     long long events = 0;
@@ -307,7 +353,17 @@ __global__ void __launch_bounds__(TAB_THREADS, 2) ev_table_batch_kernel(const __
         const lmh::TabArgs& A = B.slots[s];
         const int64_t e0 = s_eb[s] + (c - s_pre[s]) * CH;
         const Staged n = stage<lmh::EV_DATA>(A, e0, (int)min((long long)CH, s_ee[s] - e0), rec);
-        table_chunk<lmh::EV_DATA>(A, l, e0, n, rec);
+        table_chunk<lmh::EV_DATA>(A, l, e0, n, rec, &s_bad);
+    }
+    __syncthreads();
+    if (!s_bad) return;
+    for (long long c = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; c < total; c += (long long)TAB_WARPS * gridDim.x) {
+        int s = 0;
+        while (s_pre[s + 1] <= c) ++s;
+        const lmh::TabArgs& A = B.slots[s];
+        const int64_t e0 = s_eb[s] + (c - s_pre[s]) * CH;
+        const Staged n = stage<lmh::EV_DATA>(A, e0, (int)min((long long)CH, s_ee[s] - e0), rec);
+        table_again<lmh::EV_DATA>(A, l, e0, n.main, rec);
     }
 }
 

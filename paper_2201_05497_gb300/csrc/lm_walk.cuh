@@ -477,4 +477,38 @@ __device__ __forceinline__ int chunk_of(int64_t count, int64_t warps)
     return c >= 32 ? 32 : (c <= 2 ? 2 : (int)c & ~1);
 }
 
+// One x- or y-principal event pass by pass: its sum with every voxel and without
+// those of weight 0, and its back-projection without them.
+template <Tof TOF>
+__device__ __forceinline__ void forward_both(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r,
+                                             const char* __restrict__ img, float& plain, float& safe)
+{
+    plain = safe = 0.0f;
+#pragma unroll 1
+    for (int p = 0; 16 * p < (int)(r.meta & 0x7FFFu); ++p) {
+        Held t;
+        walk<1, 0, false, TOF, false, false>(l, G, P, r, p, nullptr, t);
+        if (t.off[0] == NONE) continue;
+        const float2 x = __ldg(reinterpret_cast<const float2*>(img + t.off[0]));
+        plain = fmaf(t.q1[0], x.y, fmaf(t.q0[0], x.x, plain));
+        if (t.q0[0] != 0.0f) safe = fmaf(t.q0[0], x.x, safe);
+        if (t.q1[0] != 0.0f) safe = fmaf(t.q1[0], x.y, safe);
+    }
+}
+
+template <Tof TOF>
+__device__ __forceinline__ void spread_small(const Lane& l, const Geo& G, const lmh::PairLay& P, const Rec& r, float b,
+                                             char* acc)
+{
+#pragma unroll 1
+    for (int p = 0; 16 * p < (int)(r.meta & 0x7FFFu); ++p) {
+        Held t;
+        walk<1, 0, false, TOF, false, false>(l, G, P, r, p, nullptr, t);
+        if (t.off[0] != NONE)
+            atomicAdd(reinterpret_cast<float2*>(acc + t.off[0]), make_float2(times<true>(t.q0[0], b), times<true>(t.q1[0], b)));
+    }
+}
+
+__device__ __forceinline__ bool finite(float v) { return fabsf(v) <= 3.402823466e38f; }
+
 }  // namespace lmw
