@@ -162,6 +162,7 @@ struct EvArgs {
     int u;
     const int64_t* sub_off;
     int n_subsets;
+    int64_t max_count;          // with seq: events of the largest subset
     float gamma_rho;
     unsigned* maxbits;          // float bits of max |value| (non-negative floats order as uints)
     float stepmax;

@@ -541,7 +541,15 @@ __device__ __forceinline__ void event_chunk(const EvArgs& A, const float* __rest
 // event.  Groups of G lanes then process one event each (32/G events in
 // flight per warp): lane s of a group takes planes i0 + s, i0 + s + G, ...,
 // fetching the event's parameters from the owning lane by shuffles.
-template <int MODE, bool TWO_D, int G>
+//
+// Chunks: without a queue warp w of n takes w, w + n, ...; else from the
+// launch's counter or (LOCAL) block b takes b, b + blocks, ... from a counter in
+// shared memory.  The launch's counter serves one draw (and one warp's release at
+// the end) in about 2.5 ns, so a launch of few events would wait for little
+// else (7 143 events in chunks of 1: 18 us of draws, 9 us of releases); with many
+// its draws are hidden and it evens out the blocks (launch_mode).  Two kernels,
+// because both counters in one cost 2 to 7 % in registers.
+template <int MODE, bool TWO_D, int G, bool LOCAL = false>
 __global__ void __launch_bounds__(256, G == 8 ? 2 : 3) ev_kernel(const EvArgs A)
 {
     using T = ModeTraits<MODE>;
@@ -584,28 +592,22 @@ __global__ void __launch_bounds__(256, G == 8 ? 2 : 3) ev_kernel(const EvArgs A)
     }
     float wmax = 0.0f;
     unsigned long long cnt_s = 0, cnt_t = 0;
-    // The global counter serves one draw (and one warp's release below) in about
-    // 2.5 ns, so a launch of few chunks would wait for little else (7 143 events in
-    // chunks of 1: 18 us of draws, 9 us of releases); up to eight chunks per warp
-    // block b takes the chunks b, b + blocks, ... from a counter in shared memory.
-    __shared__ int s_next;
-    const bool global_queue = A.queue != nullptr && nchunks > 8 * total_warps;
-    const bool local_queue = A.queue != nullptr && !global_queue;
-    if (local_queue) {
-        if (threadIdx.x == 0) s_next = 0;
+    __shared__ int s_next[1];
+    if (LOCAL) {
+        if (threadIdx.x == 0) s_next[0] = 0;
         __syncthreads();
     }
     int64_t it = 0;
     for (;;) {
         int64_t c;
-        if (global_queue) {
+        if (LOCAL) {
+            int k = 0;
+            if (lane == 0) k = atomicAdd(s_next, 1);
+            c = (int64_t)__shfl_sync(FULL, k, 0) * gridDim.x + blockIdx.x;
+        } else if (A.queue != nullptr) {
             unsigned long long cc = 0;
             if (lane == 0) cc = atomicAdd(A.queue, 1ULL);
             c = (int64_t)__shfl_sync(FULL, cc, 0);
-        } else if (local_queue) {
-            int k = 0;
-            if (lane == 0) k = atomicAdd(&s_next, 1);
-            c = (int64_t)__shfl_sync(FULL, k, 0) * gridDim.x + blockIdx.x;
         } else {
             c = warp_global + it * total_warps;
             ++it;
@@ -633,7 +635,7 @@ __global__ void __launch_bounds__(256, G == 8 ? 2 : 3) ev_kernel(const EvArgs A)
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
         if (lane == 0 && m > 0.0f) atomicMax(A.maxbits, __float_as_uint(m));
     }
-    if (global_queue) {
+    if (!LOCAL && A.queue != nullptr) {
         // the last warp to finish resets the counters for the next launch
         __syncwarp();
         if (lane == 0) {
@@ -751,19 +753,31 @@ __global__ void __launch_bounds__(256, G == 8 ? 2 : 3) ev_batch_kernel(const lmh
 
 size_t ev_smem(const EvArgs& a) { return a.tof_tab ? (size_t)(lmh::TOF_TAB_N + 1) * sizeof(float) : 0; }
 
+template <int MODE, bool TWO_D, int G>
+void launch_width(const EvArgs& a, int grid, cudaStream_t st)
+{
+    // The block's own counter up to 64 events per warp.  Data updates on 200 x 200 x 96 voxels, 32 lanes
+    // (3 648 warps), the launch's counter / the blocks': 20 000 events 43 / 31 us, 100 000 93 / 62, 200 000 105 / 98,
+    // 250 000 117 / 114, 357 143 152 / 156, 900 000 325 / 335.  Eight lanes keep the launch's (four events
+    // of a warp at once: 50 000 events 80 / 87 us).
+    if constexpr (G != 8 && (MODE == lmh::EV_DATA || MODE == lmh::EV_DATA_FX1 || MODE == lmh::EV_BACK_FX ||
+                             MODE == lmh::EV_YINIT || MODE == lmh::EV_YINIT_FX1 || MODE == lmh::EV_EM)) {
+        const int64_t count = a.seq ? a.max_count : a.e_end - a.e_begin;
+        if (a.queue != nullptr && count <= 64 * 8 * (int64_t)grid) {
+            ev_kernel<MODE, TWO_D, G, true><<<grid, 256, ev_smem(a), st>>>(a);
+            return;
+        }
+    }
+    ev_kernel<MODE, TWO_D, G><<<grid, 256, ev_smem(a), st>>>(a);
+}
+
 template <int MODE, bool TWO_D>
 int launch_mode(const EvArgs& a, int grid, cudaStream_t st)
 {
     switch (a.group) {
-        case 8:
-            ev_kernel<MODE, TWO_D, 8><<<grid, 256, ev_smem(a), st>>>(a);
-            break;
-        case 32:
-            ev_kernel<MODE, TWO_D, 32><<<grid, 256, ev_smem(a), st>>>(a);
-            break;
-        default:
-            ev_kernel<MODE, TWO_D, 16><<<grid, 256, ev_smem(a), st>>>(a);
-            break;
+        case 8: launch_width<MODE, TWO_D, 8>(a, grid, st); break;
+        case 32: launch_width<MODE, TWO_D, 32>(a, grid, st); break;
+        default: launch_width<MODE, TWO_D, 16>(a, grid, st); break;
     }
     lmh::count_launch();
     return cudaGetLastError() == cudaSuccess ? LM_OK : LM_ERR_CUDA;

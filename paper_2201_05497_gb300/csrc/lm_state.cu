@@ -184,6 +184,7 @@ EvArgs base_ev_args(const lm_state* st)
     a.y = st->y;
     a.sub_off = st->sub_off;
     a.n_subsets = st->n;
+    for (int k = 0; k < st->n; ++k) a.max_count = std::max(a.max_count, st->sub_off_h[k + 1] - st->sub_off_h[k]);
     a.gamma_rho = (float)(st->gamma * (double)st->P.rho);
     a.stepmax = 2.0f * std::fmax(st->g.h[0], std::fmax(st->g.h[1], st->g.h[2]));
     a.queue = st->queue;
