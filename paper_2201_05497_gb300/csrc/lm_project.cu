@@ -869,12 +869,17 @@ __device__ __forceinline__ void sens_lor(const Geo& G, int d1, int d2, float val
 // integer conversions in place of the adder's floor).  Bound by the dependent
 // read-add-write of a profile, about 20 instructions per LOR and plane with 14
 // warps per SM (the profiles take all its shared memory).
-__global__ void sens_rings_kernel(const Geo G, const float* __restrict__ lf, float* acc_std, float* acc_yf, int n_xtal,
-                                  int n_rings)
+//
+// Planes: the first P threads.  The block's other threads take part in the LORs that
+// go one by one, a warp each: 96 rings over 576 mm, 128 crystals on 150 mm (most LORs
+// z-principal) took 98.9 ms with the warps of the planes alone, 42.5 ms with them,
+// sens_kernel 42.1 ms; 72 rings 31.4, 15.5 and 23.1 ms.
+__global__ void __launch_bounds__(256, 4) sens_rings_kernel(const Geo G, const float* __restrict__ lf, float* acc_std,
+                                                            float* acc_yf, int n_xtal, int n_rings, int P)
 {
     extern __shared__ float s_dyn[];
     __shared__ int s_copies;
-    const int P = blockDim.x, R = n_rings, R2 = R * R;
+    const int T = blockDim.x, R = n_rings, R2 = R * R;
     const int nx = G.n[0], ny = G.n[1], nz = G.n[2];
     float* prof = s_dyn;                  // [nz + 4][P]: rows -2 .. nz + 1 of a plane's axial profile
     float* s_lf = prof + (nz + 4) * P;    // [R][R] LOR factors of the pair
@@ -896,14 +901,14 @@ __global__ void sens_rings_kernel(const Geo G, const float* __restrict__ lf, flo
         __syncthreads();  // the previous pair's shared data is no longer read
         if (t == 0) s_copies = 1;
         __syncthreads();
-        for (int r = t; r < R; r += P) {
+        for (int r = t; r < R; r += T) {
             const float* a = G.xtal + 3 * ((int64_t)r * n_xtal + c1);
             const float* b = G.xtal + 3 * ((int64_t)r * n_xtal + c2);
             if (a[0] != ax || a[1] != ay || b[0] != bx || b[1] != by || a[2] != b[2]) s_copies = 0;
             s_z[r] = (a[2] - oz) / hz;
             s_zr[r] = a[2];
         }
-        for (int k = t; k < R2; k += P) s_lf[k] = lf ? lf[q * R2 + k] : 1.0f;
+        for (int k = t; k < R2; k += T) s_lf[k] = lf ? lf[q * R2 + k] : 1.0f;
         __syncthreads();
         float zlo = s_zr[0], zhi = s_zr[0], zmax = 0.0f;
         for (int r = 0; r < R; ++r) {
@@ -916,7 +921,7 @@ __global__ void sens_rings_kernel(const Geo G, const float* __restrict__ lf, flo
         const float dk = k ? dy : dx, da = k ? dx : dy, adk = fabsf(dk);
         const bool copies = s_copies != 0;
         // LOR by LOR: every ring pair of the block where the rings differ, else the z-principal ones
-        const int warps = P >> 5, warp = t >> 5;
+        const int warps = T >> 5, warp = t >> 5;
         const bool z_pairs = zhi - zlo > adk;
         for (int rr = warp; rr < R2 && (!copies || z_pairs); rr += warps) {
             const int r1 = rr / R, r2 = rr - r1 * R;
@@ -935,7 +940,7 @@ __global__ void sens_rings_kernel(const Geo G, const float* __restrict__ lf, flo
             const int i = g + t;
             const float fi = (float)i;
             const float ua = fmaf(fi, sa, ua0), fla = floorf(ua), fa = ua - fla;
-            const bool in = i < nk && fla >= -1.0f && fla < (float)nA;
+            const bool in = t < P && i < nk && fla >= -1.0f && fla < (float)nA;
             if (__syncthreads_or(in) == 0) continue;
             const int ia = in ? (int)fla : 0;
             const float mu = fmaf(fi, dmu, mu0), tt = mu + 0.5f;  // position along the line from the first crystal
@@ -1610,14 +1615,25 @@ int lm_sens(const lm_scanner* sc, const lm_grid* grid, const lm_tof* tof, const 
     const int need = (std::max(grid->n[0], grid->n[1]) + 31) / 32 * 32;
     const int64_t room = 100 * 1024 - ((int64_t)R * R + 2 * R) * 4;
     const int P = (int)std::min<int64_t>(std::min(need, 256), room / ((int64_t)rows * 4) / 32 * 32);
+    const size_t smem = ((size_t)rows * std::max(P, 0) + (size_t)R * R + 2 * R) * 4;
+    int b = 0;
     if (R <= 96 && 2 * R * R > grid->n[2] && grid->n[2] >= 2 && P >= 32) {
-        const size_t smem = ((size_t)rows * P + (size_t)R * R + 2 * R) * 4;
         LM_CUDA(cudaFuncSetAttribute(sens_rings_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 101 * 1024));
-        int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, sens_rings_kernel, P, smem) != cudaSuccess || b < 1) b = 1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, sens_rings_kernel, P, smem) != cudaSuccess) b = 0;
+    }
+    // What a LOR costs: here one read-add-write chain per group of P planes, hidden by the b blocks of an SM only
+    // (about 0.47 ns of the chip's time per group over b), LOR by LOR its set-up and its planes (0.17 ns + 3.6 ps
+    // per plane).  Measured at 40 rings x 160 crystals, 20 million LORs, this against LOR by LOR: 96 x 96 x 400
+    // voxels 7.1 / 9.3 ms, x 600 (3 groups, b = 2) 10.7 / 9.4; 220 x 200 x 300 19.0 / 20.1, x 400 (7 groups,
+    // b = 3) 21.7 / 20.4, x 600 34.2 / 21.0.
+    const int planes = std::max(grid->n[0], grid->n[1]), groups = b > 0 ? (planes + P - 1) / P : 0;
+    if (b > 0 && 130 * groups <= b * (47 + planes)) {
+        // warps for the LORs that go one by one, as far as registers allow without a block fewer (64 per thread)
+        const int T = std::max(P, std::min(256, 1024 / b / 32 * 32));
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, sens_rings_kernel, T, smem) != cudaSuccess || b < 1) b = 1;
         const int64_t pairs = (int64_t)sc->n_xtal * (sc->n_xtal - 1) / 2;
         const int blocks = (int)std::min<int64_t>(pairs, (int64_t)b * num_sms());
-        sens_rings_kernel<<<blocks, P, smem, st>>>(G, lor_factor, sens, yf, sc->n_xtal, R);
+        sens_rings_kernel<<<blocks, T, smem, st>>>(G, lor_factor, sens, yf, sc->n_xtal, R, P);
         LM_CUDA(cudaGetLastError());
         count_launch();
         if (yf) launch_add_yf_to_std(grid, sens, yf, st);
