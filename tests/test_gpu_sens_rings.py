@@ -1,7 +1,8 @@
 """GPU: the sensitivity image where its rule for ring-pair profiles branches.
 A scanner longer than wide (most LORs go one by one, by warps that hold no
 planes), a grid too fine axially for the profiles (LOR by LOR throughout), against
-the FP64 oracle."""
+the FP64 oracle; and factors that are not finite, which stay with the voxels
+that their LORs touch."""
 import numpy as np
 import pytest
 
@@ -45,3 +46,18 @@ def test_sens_matches_oracle(lm, name):
     want = O.sens(geo_o, lf)
     got = lm.sens(geo, torch.from_numpy(lf).cuda()).cpu().numpy()
     assert np.linalg.norm(got - want) <= 1e-5 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_factor_stays_with_its_lor(lm, value):
+    """Rings on slice centres, so that upper neighbours weigh 0; one factor
+    that is not finite within a ring, one between two rings."""
+    sc, _, geo = geometry(lm, (9, 40, 100.0, 5.0), (24, 21, 9), 5.0, 15)
+    lf = torch.ones(sc.n_lor, device="cuda")
+    bad = torch.zeros(sc.n_lor, device="cuda")
+    for q, r1, r2 in ((18 * 40 + 7, 4, 4), (15 * 40 + 33, 1, 6)):  # nearly opposite crystals
+        bad[q * 81 + r1 * 9 + r2] = 1.0
+    touched = lm.sens(geo, bad) > 0
+    lf[bad > 0] = value
+    s = lm.sens(geo, lf)
+    assert bool(touched.any()) and bool((torch.isfinite(s) == ~touched).all())
