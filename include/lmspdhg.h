@@ -111,9 +111,9 @@ typedef struct {
 /* p_e = (P^LM x)_e = corr_e J_e(x)  (Eq. lmop).  x: device image; p: device
  * float [ev->n].  corr NULL = 1.  ws (device, may be NULL) of at least
  * lm_fwd_workspace_bytes() serves copies of x laid out for the gathers (z
- * pairs in 3D from 16384 events on, else, and with 4 bytes per voxel at least,
- * a transposed copy for y-principal events); results are the same either way
- * up to rounding. */
+ * pairs in 3D from 16384 events on, with TOF one per 256 voxels; else, and with 4
+ * bytes per voxel at least, a transposed copy for y-principal events); results
+ * are the same either way up to rounding. */
 size_t lm_fwd_workspace_bytes(const lm_grid* grid);
 int lm_fwd(const lm_scanner* sc, const lm_grid* grid, const lm_tof* tof, const float* x,
            const lm_events* ev, float* p, void* ws, size_t ws_bytes, void* stream);

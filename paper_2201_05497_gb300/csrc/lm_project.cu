@@ -1416,16 +1416,22 @@ static int operator_shape(EvArgs& a, int mode, bool two_d)
 // from WALK_EVENTS on, where its pair image (8 bytes per voxel of workspace)
 // and the table each block makes are repaid; fewer events, 2D grids, smaller
 // workspaces (4 bytes per voxel served before) and 2^29 voxels or more take the
-// event kernel.
-constexpr int64_t WALK_EVENTS = 16384;
+// event kernel.  Making the pair image costs twice the event kernel's copy, so a
+// forward projection with TOF (about 46 samples per event to win on) needs an event
+// per WALK_VOXELS voxels too.  Event kernel / walk, us: 3.8e6 voxels, 16 384 events
+// 39.5 / 40.2, 65 536 64 / 59; 31e6 voxels, 65 536 events 175 / 188, 131 072 216 /
+// 208, 1e6 771 / 499; 108e6 voxels, 16 384 events 361 / 534, 262 144 540 / 626, 524 288
+// 727 / 715.  Without TOF (16 384 events: 53 / 46, 31e6 voxels 216 / 181) and back
+// (127 / 63, 31e6 voxels 1602 / 220) the walk wins from the start.
+constexpr int64_t WALK_EVENTS = 16384, WALK_VOXELS = 256;
 
 static bool walk_grid(const lm_grid* g) { return trav_capable(g) && nvox(g) < (int64_t(1) << 29); }
 
 static size_t op_workspace(const lm_grid* g) { return align_up((size_t)nvox(g) * (walk_grid(g) ? 8 : 4)); }
 
-static bool use_walk(const lm_grid* g, int64_t n, const void* ws, size_t ws_bytes)
+static bool use_walk(const lm_grid* g, bool tof_fwd, int64_t n, const void* ws, size_t ws_bytes)
 {
-    return walk_grid(g) && n >= WALK_EVENTS && ws != nullptr && ws_bytes >= op_workspace(g) &&
+    return walk_grid(g) && n >= WALK_EVENTS && (!tof_fwd || n * WALK_VOXELS >= nvox(g)) && ws != nullptr && ws_bytes >= op_workspace(g) &&
            ((uintptr_t)ws & 15) == 0;
 }
 
@@ -1491,7 +1497,7 @@ int lm_fwd(const lm_scanner* sc, const lm_grid* grid, const lm_tof* tof, const f
     LM_CHECK(x != nullptr && p != nullptr, LM_ERR_INVALID_ARG, "x or p is NULL");
     LM_CHECK(tof->n_bins == 0 || ev->tof != nullptr, LM_ERR_INVALID_ARG, "TOF bins NULL for a TOF scanner");
     cudaStream_t st = S(stream);
-    if (use_walk(grid, ev->n, ws, ws_bytes)) {
+    if (use_walk(grid, G.tof_on != 0, ev->n, ws, ws_bytes)) {
         OpArgs o = op_args(G, grid, ev);
         launch_pair_image(grid, o.lay, x, (float*)ws, st);
         o.xp = (const float*)ws;
@@ -1549,7 +1555,7 @@ int lm_back(const lm_scanner* sc, const lm_grid* grid, const lm_tof* tof, const 
     const size_t V = (size_t)nvox(grid);
     const bool two_d = grid->n[2] == 1 && sc->n_rings == 1;  // single-ring scanner in the image plane
     const bool use_yf = grid->n[1] > 1 && ws != nullptr && ws_bytes >= need;
-    if (!deterministic && use_walk(grid, ev->n, ws, ws_bytes)) {
+    if (!deterministic && use_walk(grid, false, ev->n, ws, ws_bytes)) {
         OpArgs o = op_args(G, grid, ev);
         o.v = v;
         o.acc = (float*)ws;
