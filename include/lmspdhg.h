@@ -282,12 +282,16 @@ typedef struct {
     int32_t kahan;        /* 1: compensated float32 accumulation of z             */
     int32_t group;        /* lanes per event in the event kernels: 8, 16 or 32;  */
                           /* 0: chosen at create by timing the forward projection */
-                          /* of subset 0 with each width (autotuner)             */
+                          /* of subset 0 with each width (autotuner; with         */
+                          /* trav_buf the direct kernel's data update of it)      */
     int32_t image_kernel; /* image passes: 0 auto (TMA-staged where the grid has */
                           /* nx, ny multiples of 4, nx >= 40, ny >= 36, with the  */
                           /* TV's dual step fused in, the directional TV's D =    */
-                          /* P(w+ - w) staged from its dual step; plain loads     */
-                          /* otherwise), 1 plain loads, 2 TMA-staged, 3 TMA-      */
+                          /* P(w+ - w) staged from its dual step; one voxel per   */
+                          /* thread with the dual step fused in for 2D grids of   */
+                          /* at most 2^17 voxels in float-atomic mode with the    */
+                          /* TV, except in batches; plain loads otherwise), 1     */
+                          /* plain loads, 2 TMA-staged, 3 TMA-      */
                           /* staged data passes with plain prior passes (2 and 3: */
                           /* LM_ERR_INVALID_ARG if the grid does not allow it;    */
                           /* other values: LM_ERR_INVALID_ARG).  Same results.    */
@@ -332,12 +336,16 @@ typedef struct {
                           /* ignored.  At create/reinit every event's traversal  */
                           /* (the reading of Joseph's method: principal axis,    */
                           /* plane range, secondary and TOF coordinates, sample  */
-                          /* length), 1/(P^LM 1)_e and 1/mu_e are stored (40 B   */
+                          /* length), 1/(P^LM 1)_e and mu_e are stored (40 B     */
                           /* per event); each data update then reads them        */
                           /* instead of setting the traversals up again, walking  */
                           /* z-pair copies of x (two lanes per voxel plane,       */
                           /* whatever `group` says).  Same samples and weights as */
-                          /* the direct kernel, summed in another order; S_e and  */
+                          /* the direct kernel, summed in another order (samples  */
+                          /* within an ulp of the n_sigma cut, a few per 1e6      */
+                          /* events, are decided by another rounding of the TOF   */
+                          /* coordinate, except with group = 0, trav_keep = 0 and */
+                          /* fewer than 65536 events in the first subset); S_e and*/
                           /* (y+ - y)/mu from stored values.  Grids of 2^29       */
                           /* voxels or more use the direct kernel.  Batches       */
                           /* (lmspdhg_batch_*) run their frames' tables too.     */
@@ -442,8 +450,10 @@ int lmspdhg_objective_fp64(lm_state* st, double* out_host, void* stream);
  * as resolved at create). */
 int lmspdhg_info(lm_state* st, int64_t* n_updates, double* gamma, double* knorm);
 
-/* The event-kernel width in use and, if it was autotuned, the measured
- * forward-projection times of subset 0 (ms) for widths 8, 16, 32 (else 0). */
+/* The event-kernel width in use and, if it was autotuned, the times (ms) of
+ * subset 0 measured for widths 8, 16, 32: forward projections, or with
+ * lm_params.trav_buf the direct kernel's data updates (else 0; 0 with
+ * trav_keep). */
 int lmspdhg_tuning(lm_state* st, int32_t* group, double* ms3);
 
 /* Re-initialise the state (as lmspdhg_create initialises Alg. 2) for the
@@ -494,8 +504,8 @@ int lmspdhg_shard_finish(lm_state* st, void* stream);
 int lmspdhg_objective_parts_fp64(lm_state* st, double* out4, void* stream);
 
 /* The autotuner's comparison of the projectors (lm_params.trav_buf with
- * group = 0): the data update of subset 0 with the best traversal-table
- * variant and with the best direct-kernel width, in ms (0 when not
+ * group = 0): the data update of subset 0 with the traversal table
+ * and with the best direct-kernel width, in ms (0 when not
  * measured); the state keeps the faster one (lmspdhg_projector), or the
  * table when lm_params.trav_keep is set (the direct kernel is then not
  * timed and direct_ms is 0). */
@@ -514,7 +524,7 @@ int lmspdhg_set_gate(lm_state* st, const unsigned* flag);
 int lmspdhg_epoch_kernel(lm_state* st, int32_t* kind);
 
 /* Which image-pass kernel the state uses (lm_params.image_kernel): 1 plain
- * loads, 2 TMA-staged (the TV's dual step fused in; the directional TV's
+ * loads (also the one-voxel-per-thread passes of small 2D grids), 2 TMA-staged (the TV's dual step fused in; the directional TV's
  * dual step stays in the event kernel and the pass stages its D), 3
  * TMA-staged data passes with plain prior passes. */
 int lmspdhg_image_kernel(lm_state* st, int32_t* kind);

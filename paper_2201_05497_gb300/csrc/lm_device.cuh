@@ -49,8 +49,8 @@ __device__ __forceinline__ int sel3i(int k, int a, int b, int c) { return k == 0
 
 // Sets up the traversal; returns false if the LOR has no candidate sample.
 // m: signed TOF bin (ignored unless tofmode == TOF_BIN).
-// stored: the traversal is kept (tables, tiles) rather than used at once; it
-// only chooses which product of the TOF coordinate is rounded first.
+// stored: the rounding of the traversal tables and tiles; it only chooses
+// which product of the TOF coordinate is rounded first.
 __device__ __forceinline__ bool lor_setup(const Geo& G, int d1, int d2, int m, int tofmode, bool has_yf,
                                           Lor& L, bool stored = false)
 {

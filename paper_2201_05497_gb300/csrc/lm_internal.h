@@ -322,7 +322,7 @@ struct PairLay {
 PairLay pair_layout(const lm_grid* g, bool rows);  // rows: no bricks even where the grid allows them
 
 // Per event (subset-contiguous order): the traversal of reading 1,
-// 1/(P^LM 1)_e and 1/mu_e, computed once per state.
+// 1/(P^LM 1)_e and mu_e, computed once per state.
 struct TravLayout {
     size_t r0, r1, meta, total;
 };
@@ -338,7 +338,6 @@ struct TabArgs {
     // events
     const float* corr;
     const float* contam;
-    const uint16_t* mu;
     float* y;
     // images as z pairs (voxel j, voxel j + nx*ny): the x the events read, the accumulator
     const float* xp;

@@ -1519,7 +1519,6 @@ int lm_fwd(const lm_scanner* sc, const lm_grid* grid, const lm_tof* tof, const f
     a.out = p;
     a.e_begin = 0;
     a.e_end = ev->n;
-    a.chunk = 32;
     const bool two_d = grid->n[2] == 1 && sc->n_rings == 1;  // single-ring scanner in the image plane
     const int blocks = operator_shape(a, EV_FWD, two_d);
     rc = launch_events(EV_FWD, two_d, a, blocks, st);

@@ -278,7 +278,6 @@ TabArgs base_tab_args(const lm_state* st)
     t.meta = (const int2*)(st->tv_base + st->tv.meta);
     t.corr = st->corr;
     t.contam = st->contam;
-    t.mu = st->mu;
     t.y = st->y;
     t.xp = pair_image(st);
     t.acc = st->acc_std;
@@ -301,10 +300,11 @@ int build_table(lm_state* st, cudaStream_t s)
     ev.corr = st->corr;
     ev.contam = st->contam;
     ev.n = st->N;
-    // Which product of the TOF coordinate is rounded first (lor_setup) moves samples within an ulp of the
-    // 3-sigma cut in or out of the window, a few per 1e6 events.  Small updates of frames that leave the
-    // projector open ran the direct kernel (it was the faster one below about 64 000 events), all others the
-    // table: each keeps the samples it had.
+    // Which product of the TOF coordinate is rounded first (lor_setup) decides on samples within an ulp of the
+    // cut, a few per 1e6 events.  Neither is nearer to the exact line, but the iterates carry it: up to 1e-2 of the
+    // largest w after an epoch, 1e-5 of x.  Where the projector is open and the timing may go either way (updates
+    // of fewer than 65 536 events) the table takes the direct kernel's rounding, so that the timing's outcome
+    // does not move a frame's samples; frames that keep the table and larger ones, where it always wins, have its own.
     const bool stored = st->P.group != 0 || st->P.trav_keep || st->sub_off_h[1] - st->sub_off_h[0] >= 65536;
     return trav_build(st->G, ev, st->mu, st->tof_tab, st->tv, st->tv_base, stored, s);
 }

@@ -9,17 +9,17 @@
 // and mu_e once per state (trav_build), so a data update reads 40 bytes of
 // table per event, and walks the events over z-pair images (lm_walk.cuh).
 //
-// Measured on the 200 x 200 x 96 grid (GB300, CUDA events around the launch),
-// one plane per lane over two image layouts and two accumulators (before) /
-// two lanes per plane over bricked z pairs: 7 143 events 17.5 / 14.1 us,
-// 357 143 events 200 / 133 us, 2.14e6 events 1.09 ms / 0.67 ms.  ncu at
-// 357 143 events: with the pairs in rows 71 % of the SM-to-L2 request cycles
-// (17.1 M lines gathered + 19.5 M sectors added to), issue 42 %, 176 us; in bricks
-// 9.2 M + 16.0 M, request cycles 65 %, issue 72 % (305 warp instructions per
-// event), 133 us: instructions and requests now bound it about equally.
+// Measured on the 200 x 200 x 96 grid (GB300, CUDA events around the launch,
+// Monte Carlo events): 7 143 events 14.5 us, 50 000 33 us, 357 143 136 us, 1.07e6
+// 356 us; one plane per lane over two image layouts and two accumulators took 200 us
+// at 357 143.  ncu at 357 143 events: with the pairs in rows 71 % of the SM-to-L2
+// request cycles (17.1 M lines gathered + 19.5 M sectors added to), issue 42 %, 176
+// us; in bricks 9.2 M + 16.0 M: instructions and requests now bound it about
+// equally (profiles/ev_table_kernel_data_update_3d_short.txt).
 // Ordering the events by direction and place moved it by less than 10 % in
 // either direction, and one-plane-per-lane with the same pairs was no faster.
-// Per sample the positions and weights are the direct kernel's.
+// Per sample the positions and weights are the direct kernel's (lor_setup; see
+// build_table for the rounding of the TOF coordinate).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
