@@ -1431,8 +1431,8 @@ static size_t op_workspace(const lm_grid* g) { return align_up((size_t)nvox(g) *
 
 static bool use_walk(const lm_grid* g, bool tof_fwd, int64_t n, const void* ws, size_t ws_bytes)
 {
-    return walk_grid(g) && n >= WALK_EVENTS && (!tof_fwd || n * WALK_VOXELS >= nvox(g)) && ws != nullptr && ws_bytes >= op_workspace(g) &&
-           ((uintptr_t)ws & 15) == 0;
+    return walk_grid(g) && n >= WALK_EVENTS && (!tof_fwd || n * WALK_VOXELS >= nvox(g)) && ws != nullptr &&
+           ws_bytes >= op_workspace(g) && ((uintptr_t)ws & 15) == 0;
 }
 
 static OpArgs op_args(const lmk::Geo& G, const lm_grid* g, const lm_events* ev)
