@@ -756,14 +756,17 @@ size_t ev_smem(const EvArgs& a) { return a.tof_tab ? (size_t)(lmh::TOF_TAB_N + 1
 template <int MODE, bool TWO_D, int G>
 void launch_width(const EvArgs& a, int grid, cudaStream_t st)
 {
-    // The block's own counter up to 64 events per warp.  Data updates on 200 x 200 x 96 voxels, 32 lanes
+    // The block's own counter up to 8 chunks per warp, in data updates up to 64 events per warp (their chunks
+    // grow with the events; EM steps and the initialisation lose nothing by it: EM step of 500 000 events
+    // 743 / 737 us, and its fixed blocks vary the order of the float sums less).  Data updates on 200 x 200 x 96 voxels, 32 lanes
     // (3 648 warps), the launch's counter / the blocks': 20 000 events 43 / 31 us, 100 000 93 / 62, 200 000 105 / 98,
     // 250 000 117 / 114, 357 143 152 / 156, 900 000 325 / 335.  Eight lanes keep the launch's (four events
     // of a warp at once: 50 000 events 80 / 87 us).
     if constexpr (G != 8 && (MODE == lmh::EV_DATA || MODE == lmh::EV_DATA_FX1 || MODE == lmh::EV_BACK_FX ||
                              MODE == lmh::EV_YINIT || MODE == lmh::EV_YINIT_FX1 || MODE == lmh::EV_EM)) {
-        const int64_t count = a.seq ? a.max_count : a.e_end - a.e_begin;
-        if (a.queue != nullptr && count <= 64 * 8 * (int64_t)grid) {
+        const int64_t count = a.seq ? a.max_count : a.e_end - a.e_begin, warps = 8 * (int64_t)grid;
+        const bool data = MODE == lmh::EV_DATA || MODE == lmh::EV_DATA_FX1;
+        if (a.queue != nullptr && (count + a.chunk - 1) / a.chunk <= 8 * warps && (!data || count <= 64 * warps)) {
             ev_kernel<MODE, TWO_D, G, true><<<grid, 256, ev_smem(a), st>>>(a);
             return;
         }

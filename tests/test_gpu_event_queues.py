@@ -1,6 +1,6 @@
-"""GPU: the event kernel's two work counters.  Launches of up to 64 events per
-warp (16 and 32 lanes per event) draw their chunks from a counter per block,
-larger ones and 8 lanes from the launch's; both sides of the line give the same
+"""GPU: the event kernel's two work counters.  Launches of up to eight chunks per
+warp (data updates: 64 events; 16 and 32 lanes per event) draw them from a counter
+per block, larger ones and 8 lanes from the launch's; both sides of the line give the same
 sums to rounding."""
 import numpy as np
 import pytest
@@ -52,15 +52,15 @@ def test_data_updates_agree_over_widths(lm, two_d, n_ev):
 
 @pytest.mark.parametrize("two_d", [False, True])
 def test_em_step_equals_its_parts(lm, two_d):
-    """The EM back-projection is a sum over events: of 300 000 in one launch, of
-    60 000 in each of five."""
-    geo, ev = frame(lm, two_d, 300000)
+    """The EM back-projection is a sum over events: of 1 000 000 in one launch, of
+    200 000 in each of five."""
+    geo, ev = frame(lm, two_d, 1000000)
     rng = np.random.default_rng(4)
     sens = torch.from_numpy(rng.uniform(1, 2, geo.V).astype(np.float32)).cuda()
     x = torch.from_numpy(rng.uniform(0.5, 1.5, geo.V).astype(np.float32)).cuda()
     whole = lm.emtv_em_step(geo, ev, 1, sens, x).double()
     parts = torch.zeros_like(whole)
-    for s in range(0, ev.n, 60000):
-        part = lm.DeviceEvents(*[t[s:s + 60000].contiguous() for t in (ev.det1, ev.det2, ev.tof, ev.corr, ev.contam)])
+    for s in range(0, ev.n, 200000):
+        part = lm.DeviceEvents(*[t[s:s + 200000].contiguous() for t in (ev.det1, ev.det2, ev.tof, ev.corr, ev.contam)])
         parts += lm.emtv_em_step(geo, part, 1, sens, x).double()
     assert float((whole - parts).norm() / parts.norm()) < 2e-6
