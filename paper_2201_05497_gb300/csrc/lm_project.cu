@@ -869,7 +869,7 @@ __device__ __forceinline__ void sens_lor(const Geo& G, int d1, int d2, float val
 // copies, and LORs with a factor that is not finite (whose samples of weight 0 must
 // not enter a profile) go LOR by LOR as in sens_kernel.
 // Measured on 36 x 672 crystals, 200 x 200 x 96 voxels (2.9e8 LORs): sens_kernel
-// (bound by its 4 atomics per sample) 248 ms, this 77.6 ms (87 ms with float to
+// (bound by its 4 atomics per sample) 248 ms, this 75.8 ms (87 ms with float to
 // integer conversions in place of the adder's floor).  Bound by the dependent
 // read-add-write of a profile, about 20 instructions per LOR and plane with 14
 // warps per SM (the profiles take all its shared memory).
@@ -878,8 +878,8 @@ __device__ __forceinline__ void sens_lor(const Geo& G, int d1, int d2, float val
 // go one by one, a warp each: 96 rings over 576 mm, 128 crystals on 150 mm (most LORs
 // z-principal) took 98.9 ms with the warps of the planes alone, 42.5 ms with them,
 // sens_kernel 42.1 ms; 72 rings 31.4, 15.5 and 23.1 ms.
-__global__ void __launch_bounds__(256, 4) sens_rings_kernel(const Geo G, const float* __restrict__ lf, float* acc_std,
-                                                            float* acc_yf, int n_xtal, int n_rings, int P)
+__global__ void __launch_bounds__(256) sens_rings_kernel(const Geo G, const float* __restrict__ lf, float* acc_std,
+                                                         float* acc_yf, int n_xtal, int n_rings, int P)
 {
     extern __shared__ float s_dyn[];
     __shared__ int s_copies;
@@ -912,22 +912,20 @@ __global__ void __launch_bounds__(256, 4) sens_rings_kernel(const Geo G, const f
             s_z[r] = (a[2] - oz) / hz;
             s_zr[r] = a[2];
         }
+        for (int k = t; k < R2; k += T) s_lf[k] = lf ? lf[q * R2 + k] : 1.0f;
+        // factors that are not finite: taken out here, their LORs one by one below
         bool not_finite = false;
-        for (int k0 = t; k0 < R2; k0 += 8 * T) {  // eight loads in flight
-            float f[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) f[e] = lf && k0 + e * T < R2 ? __ldg(lf + q * R2 + k0 + e * T) : 1.0f;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                not_finite |= !(fabsf(f[e]) <= 3.402823466e38f);
-                if (k0 + e * T < R2) s_lf[k0 + e * T] = f[e];
+        for (int k = t; k < R2; k += T)
+            if (!(fabsf(s_lf[k]) <= 3.402823466e38f)) {
+                s_lf[k] = 0.0f;
+                not_finite = true;
             }
-        }
-        const bool odd = __syncthreads_or(not_finite) != 0;
-        if (odd) {
-            for (int k = t; k < R2; k += T)
-                if (!(fabsf(s_lf[k]) <= 3.402823466e38f)) s_lf[k] = 0.0f;
-            __syncthreads();
+        if (__syncthreads_or(not_finite)) {
+            for (int rr = t >> 5; rr < R2; rr += T >> 5) {
+                const float f = lf[q * R2 + rr];
+                const int r1 = rr / R, r2 = rr - r1 * R;
+                if (!(fabsf(f) <= 3.402823466e38f)) sens_lor(G, r1 * n_xtal + c1, r2 * n_xtal + c2, f, acc_std, acc_yf);
+            }
         }
         float zlo = s_zr[0], zhi = s_zr[0], zmax = 0.0f;
         for (int r = 0; r < R; ++r) {
@@ -939,14 +937,13 @@ __global__ void __launch_bounds__(256, 4) sens_rings_kernel(const Geo G, const f
         const int k = fabsf(dy) > fabsf(dx) ? 1 : 0;
         const float dk = k ? dy : dx, da = k ? dx : dy, adk = fabsf(dk);
         const bool copies = s_copies != 0;
-        // LOR by LOR: every ring pair of the block where the rings differ, else the z-principal and the odd ones
+        // LOR by LOR: every ring pair of the block where the rings differ, else the z-principal ones
         const int warps = T >> 5, warp = t >> 5;
         const bool z_pairs = zhi - zlo > adk;
-        for (int rr = warp; rr < R2 && (!copies || z_pairs || odd); rr += warps) {
+        for (int rr = warp; rr < R2 && (!copies || z_pairs); rr += warps) {
             const int r1 = rr / R, r2 = rr - r1 * R;
-            const float f = odd ? lf[q * R2 + rr] : s_lf[rr];
-            if (copies && !(fabsf(s_zr[r2] - s_zr[r1]) > adk) && fabsf(f) <= 3.402823466e38f) continue;
-            sens_lor(G, r1 * n_xtal + c1, r2 * n_xtal + c2, f, acc_std, acc_yf);
+            if (copies && !(fabsf(s_zr[r2] - s_zr[r1]) > adk)) continue;
+            sens_lor(G, r1 * n_xtal + c1, r2 * n_xtal + c2, s_lf[rr], acc_std, acc_yf);
         }
         if (!copies || adk == 0.0f) continue;
         const int nk = k ? ny : nx, nA = k ? nx : ny;
@@ -1653,8 +1650,9 @@ int lm_sens(const lm_scanner* sc, const lm_grid* grid, const lm_tof* tof, const 
     // b = 3) 21.7 / 20.4, x 600 34.2 / 21.0.
     const int planes = std::max(grid->n[0], grid->n[1]), groups = b > 0 ? (planes + P - 1) / P : 0;
     if (b > 0 && 130 * groups <= b * (47 + planes)) {
-        // warps for the LORs that go one by one, as far as registers allow without a block fewer (64 per thread)
-        const int T = std::max(P, std::min(256, 1024 / b / 32 * 32));
+        // warps for the LORs that go one by one, as far as registers allow without a block fewer (about 64 per
+        // thread); where the planes alone bring 16 warps to an SM, idle ones would only cost (2 to 6 %)
+        const int T = b * P >= 512 ? P : std::max(P, std::min(256, 1024 / b / 32 * 32));
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, sens_rings_kernel, T, smem) != cudaSuccess || b < 1) b = 1;
         const int64_t pairs = (int64_t)sc->n_xtal * (sc->n_xtal - 1) / 2;
         const int blocks = (int)std::min<int64_t>(pairs, (int64_t)b * num_sms());
